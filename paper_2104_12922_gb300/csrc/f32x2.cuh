@@ -1,0 +1,39 @@
+// f32x2.cuh -- pairs of floats in one 64-bit register: Blackwell's packed FP32
+// add, multiply and fused multiply-add. A packed instruction keeps the FP32
+// pipe busy as long as two scalar ones (measured: 1.97 a clock and SM against
+// 3.85) but takes one issue slot, so it pays where instruction issue is what
+// runs out. Each half rounds as the scalar instruction does.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace synth {
+
+typedef unsigned long long f32x2;
+
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 both2(float a) { return pack2(a, a); }
+__device__ __forceinline__ void unpack2(f32x2 p, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(p));
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+}  // namespace synth
