@@ -49,6 +49,8 @@ constexpr int P = kFusedTilePoints;
 constexpr int TI = kFusedTileSeg;
 constexpr int kWarps = NT / 32;
 static_assert(NT == P, "one thread per control point");
+constexpr int kCtasPerSm = 4;
+constexpr int kMaxParts = 8;  // CTAs that share a tile (kSplit)
 
 using u64 = unsigned long long;
 
@@ -275,15 +277,26 @@ __device__ __forceinline__ void release_next_launch(bool& released) {
   released = true;
 }
 
-template <bool kCarryF32, bool kPeak, bool kGenR>
-__global__ void __launch_bounds__(NT, 4) render_fused_kernel(
+// kSplit: a launch whose tiles are all resident at once (86 voices of 4 s, or
+// fewer). Where they leave SMs empty, `parts` CTAs share a tile: each runs the
+// control steps in full and renders its share of the tile's intervals, the
+// first alone publishes the tile's aggregates and the parameters. And the next
+// launch is released between a tile's control steps and its VCO intervals, not
+// at its start: the wait for the previous launch that comes with it would keep
+// every tile of this one from starting, where with it in the middle two
+// launches in a row overlap. One 4 s voice a launch, launches in a row: 28.0 ->
+// 11.7 us (alone 32.4 -> 24.3), 8 voices 31.2 -> 17.7, 16: 35.2 -> 27.3, 32: 44.1
+// -> 35.2, 64: 58.0 -> 42.6, 80: 62.4 -> 51.7.
+template <bool kCarryF32, bool kPeak, bool kGenR, bool kSplit>
+__global__ void __launch_bounds__(NT, kCtasPerSm) render_fused_kernel(
     const __grid_constant__ VoiceConst vc, uint64_t seed, uint64_t first, int split, int batch,
     const float* __restrict__ params_in, float* __restrict__ audio, float* __restrict__ params_out,
     ScratchHeader* hdr, TileState* tiles, int n_windows, const PeakNormArgs norm,
-    uint64_t seed_step, int sub_batch, VoiceSetupRecord* setups) {
+    uint64_t seed_step, int sub_batch, VoiceSetupRecord* setups, int parts) {
   __shared__ Smem s;
   const int tid = threadIdx.x;
   const int total_tiles = batch * n_windows;
+  static_assert(!kSplit || !kPeak, "a tile's peak is one CTA's");
   const int R = vc.R, K = vc.K;
   const int64_t N = vc.n_samples;
   const int qps = R >> 2;             // quads per control interval
@@ -309,7 +322,8 @@ __global__ void __launch_bounds__(NT, 4) render_fused_kernel(
       s.setup_ready = ready;
     }
     __syncthreads();  // also: the previous tile's audio is done with the shared buffers
-    const int t = s.tile;
+    const int t = kSplit ? s.tile / parts : s.tile;
+    const int part = kSplit ? s.tile - t * parts : 0;
     if (t >= total_tiles) {
       // peak variant: the scaling chunks follow the render tiles, voice by
       // voice (window-major tiles finish their voices in that order)
@@ -323,7 +337,8 @@ __global__ void __launch_bounds__(NT, 4) render_fused_kernel(
       if (t + (int)gridDim.x >= total_items) release_next_launch(released);
       continue;
     }
-    if (t + (int)gridDim.x >= total_items) release_next_launch(released);  // likely the last tile
+    if (!kSplit && t + (int)gridDim.x >= total_items)
+      release_next_launch(released);  // likely the last tile
     const int v = t % batch, w = t / batch;
     // the tile's voice and window address its set-up, tile and output records
     if (!in_bounds(hdr, v, batch) || !in_bounds(hdr, w, n_windows)) continue;
@@ -367,7 +382,7 @@ __global__ void __launch_bounds__(NT, 4) render_fused_kernel(
       __syncthreads();
       if (tid < kNumParams) {
         const float u = s.u[tid];
-        if (w == 0 && params_out &&
+        if (w == 0 && part == 0 && params_out &&
             in_bounds(hdr, (long long)v * kNumParams + tid, (long long)batch * kNumParams))
           params_out[(size_t)v * kNumParams + tid] = u;
         s.y[tid] = range_map_ff(u, vc.map_base[tid], vc.map_scale[tid], vc.map_curve[tid],
@@ -428,7 +443,7 @@ __global__ void __launch_bounds__(NT, 4) render_fused_kernel(
     {
       u64 t0, t1;
       block_scan2_fix(r0, r1, s.warp_tot[0], t0, t1);
-      if (tid == 0) lookback_publish<u64>(vt, w, 0, epoch, t0, t1);
+      if (tid == 0 && part == 0) lookback_publish<u64>(vt, w, 0, epoch, t0, t1);
       if (has_pt) {
 #pragma unroll 1
         for (int i = 0; i < 4; ++i) {  // envelopes 0, 1, 3, 5
@@ -478,6 +493,8 @@ __global__ void __launch_bounds__(NT, 4) render_fused_kernel(
       cuda::atomic_ref<unsigned int, cuda::thread_scope_device> f(setups[v].flag);
       f.store(((epoch & 0x3fffffffu) << 2) | 1u, cuda::memory_order_release);
     }
+
+    if (kSplit) release_next_launch(released);
 
     // ---- 4. VCO phase over each control interval, scanned -----------------
     ff tot[2] = {ff_make(0.f), ff_make(0.f)};
@@ -541,7 +558,8 @@ __global__ void __launch_bounds__(NT, 4) render_fused_kernel(
       block_scan2_fix(c0, c1, s.warp_tot[1], t0, t1);
       if (tid < 32) {
         u64 e0, e1;
-        lookback<u64>(vt, w, 1, epoch, t0, t1, e0, e1, hdr);
+        if (tid == 0 && part == 0) lookback_publish<u64>(vt, w, 1, epoch, t0, t1);
+        lookback_consume<u64>(vt, w, 1, epoch, e0, e1, hdr);
         if (tid == 0) { s.prefix[1][0] = e0; s.prefix[1][1] = e1; }
       }
       __syncthreads();
@@ -570,6 +588,9 @@ __global__ void __launch_bounds__(NT, 4) render_fused_kernel(
     __syncthreads();
 
     // ---- 5. audio ----------------------------------------------------------
+    // this CTA's share of the tile's intervals
+    const int seg0 = kSplit ? nseg * part / parts : 0;
+    const int seg1 = kSplit ? nseg * (part + 1) / parts : nseg;
     if constexpr (kGenR) {
       // fractional R: quads of the voice's own 4-sample grid. A work item is
       // (interval, chunk): the quad that straddles the interval's start is
@@ -659,7 +680,7 @@ __global__ void __launch_bounds__(NT, 4) render_fused_kernel(
       // first the quads that straddle an interval's start (or the tile's
       // start or end), one loop of their own so that the run loop below
       // carries none of their state
-      for (int si = tid; si < nseg; si += NT) {
+      for (int si = seg0 + tid; si < seg1; si += NT) {
         const int a = s.sst[si], b = s.sst[si + 1];
         const int f = a + (int)((-(s_tile + a)) & 3);  // first grid quad at or after a
         const int nf = b - f >= 4 ? (b - f) >> 2 : 0;   // quads wholly inside [a, b)
@@ -672,7 +693,7 @@ __global__ void __launch_bounds__(NT, 4) render_fused_kernel(
       constexpr int kGenG = 5;
       const int full_max = (int)(vc.r_f * 0.25f) + 2;  // bound on an interval's whole quads
       const int cpi = (full_max + kGenG - 1) / kGenG;   // chunks per interval
-      for (int it = tid; it < nseg * cpi; it += NT) {
+      for (int it = seg0 * cpi + tid; it < seg1 * cpi; it += NT) {
         const int si = it / cpi, c = it - si * cpi;
         const int a = s.sst[si], b = s.sst[si + 1];
         const int f = a + (int)((-(s_tile + a)) & 3);
@@ -745,9 +766,9 @@ __global__ void __launch_bounds__(NT, 4) render_fused_kernel(
       // has not got).
       const int G = qps % 5 == 0 ? 5 : qps % 4 == 0 ? 4 : qps % 3 == 0 ? 3 : qps % 2 == 0 ? 2 : 1;
       const int gpi = qps / G;
-      const int ngr = nseg * gpi;
+      const int ngr = seg1 * gpi;
       float vmax = 0.f;  // largest |sample| this thread wrote (kPeak)
-      for (int gi = tid; gi < ngr; gi += NT) {
+      for (int gi = seg0 * gpi + tid; gi < ngr; gi += NT) {
         const int si = gi / gpi;
         const int j0 = (gi - si * gpi) * (4 * G);  // the run's first sample in its interval
         const int off0 = si * R + j0;
@@ -898,7 +919,7 @@ void note_early_release_launch(cudaStream_t st) {
 
 int fused_max_active_blocks_per_sm() {
   int n = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, render_fused_kernel<false, false, false>, NT, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, render_fused_kernel<false, false, false, false>, NT, 0);
   return n;
 }
 
@@ -910,7 +931,15 @@ cudaError_t launch_render_fused(const VoiceConst& vc, uint64_t seed, uint64_t fi
                                 void* voice_setups) {
   const int n_windows = windows_per_voice(vc.K);
   const int total = batch * n_windows;
-  grid = grid < total ? grid : total;
+  // a launch whose tiles are all resident at once; where they leave SMs empty,
+  // each tile goes to as many CTAs as give every SM one (a second CTA on an SM
+  // slows the first one's control steps by more than it saves), at most
+  // kMaxParts (beyond, the copies of the control steps no longer pay)
+  const bool shared = !norm && !vc.carry_fp32 && total <= grid;
+  int parts = shared ? grid / kCtasPerSm / total : 1;
+  parts = parts < 1 ? 1 : parts < kMaxParts ? parts : kMaxParts;
+  if (parts > 1) voice_setups = nullptr;  // no window starts after another has finished
+  grid = grid < total * parts ? grid : total * parts;
   const PeakNormArgs nz = norm ? *norm : PeakNormArgs{0.f, nullptr, nullptr};
   if (sub_batch <= 0) sub_batch = batch;
   cudaLaunchConfig_t cfg = {};
@@ -941,17 +970,19 @@ cudaError_t launch_render_fused(const VoiceConst& vc, uint64_t seed, uint64_t fi
   cfg.numAttrs = overlap ? 1 : 0;
   VoiceSetupRecord* setups = static_cast<VoiceSetupRecord*>(voice_setups);
 #define SYNTH_FUSED_ARGS vc, seed, first, split, batch, params_in, audio, params_out, hdr, tiles, \
-                         n_windows, nz, seed_step, sub_batch, setups
+                         n_windows, nz, seed_step, sub_batch, setups, parts
   cudaError_t e;
   if (vc.general_r) {  // fractional R (never with FP32 carries)
-    if (norm) e = cudaLaunchKernelEx(&cfg, render_fused_kernel<false, true, true>, SYNTH_FUSED_ARGS);
-    else e = cudaLaunchKernelEx(&cfg, render_fused_kernel<false, false, true>, SYNTH_FUSED_ARGS);
+    if (norm) e = cudaLaunchKernelEx(&cfg, render_fused_kernel<false, true, true, false>, SYNTH_FUSED_ARGS);
+    else if (shared) e = cudaLaunchKernelEx(&cfg, render_fused_kernel<false, false, true, true>, SYNTH_FUSED_ARGS);
+    else e = cudaLaunchKernelEx(&cfg, render_fused_kernel<false, false, true, false>, SYNTH_FUSED_ARGS);
   } else if (vc.carry_fp32) {
-    if (norm) e = cudaLaunchKernelEx(&cfg, render_fused_kernel<true, true, false>, SYNTH_FUSED_ARGS);
-    else e = cudaLaunchKernelEx(&cfg, render_fused_kernel<true, false, false>, SYNTH_FUSED_ARGS);
+    if (norm) e = cudaLaunchKernelEx(&cfg, render_fused_kernel<true, true, false, false>, SYNTH_FUSED_ARGS);
+    else e = cudaLaunchKernelEx(&cfg, render_fused_kernel<true, false, false, false>, SYNTH_FUSED_ARGS);
   } else {
-    if (norm) e = cudaLaunchKernelEx(&cfg, render_fused_kernel<false, true, false>, SYNTH_FUSED_ARGS);
-    else e = cudaLaunchKernelEx(&cfg, render_fused_kernel<false, false, false>, SYNTH_FUSED_ARGS);
+    if (norm) e = cudaLaunchKernelEx(&cfg, render_fused_kernel<false, true, false, false>, SYNTH_FUSED_ARGS);
+    else if (shared) e = cudaLaunchKernelEx(&cfg, render_fused_kernel<false, false, false, true>, SYNTH_FUSED_ARGS);
+    else e = cudaLaunchKernelEx(&cfg, render_fused_kernel<false, false, false, false>, SYNTH_FUSED_ARGS);
   }
 #undef SYNTH_FUSED_ARGS
   if (e != cudaSuccess) return e;
