@@ -197,8 +197,10 @@ __device__ __forceinline__ GemmItem gemm_item(int item, int n_tiles, int tiles_n
 
 // part == nullptr: the epilogue `epi` is applied to each finished tile.
 // Otherwise (split-K, `splits` slices of kb_per k-blocks each) the raw
-// accumulator of slice s goes to part[s][M][N].
-template <int BN>
+// accumulator of slice s goes to part[s][M][N]. kGate: the unsplit product of
+// kEpiReluGradBF16 (an instantiation of its own, which leaves the others'
+// epilogue as it is).
+template <int BN, bool kGate>
 __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tc(
     const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
     GemmEpilogue epi, int M, int N, int K, int splits, int kb_per, float* part,
@@ -298,13 +300,31 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tc(
       if (!ok) { sm.failed = 1; break; }
       const int row0 = g.m0 + 32 * q;
       const uint32_t acc = tmem + (uint32_t)(buf * BN) + ((uint32_t)(32 * q) << 16);
-      const bool act = !part && epi.kind == kEpiBiasActBF16;
+      const bool act = kGate || (!part && epi.kind == kEpiBiasActBF16);
 #pragma unroll 1
       for (int c = half * (BN / 2); c < (half + 1) * (BN / 2); c += 32) {
         float v[32];
         tmem_ld32(acc + (uint32_t)c, v);
         const int col0 = g.n0 + c;
-        if (act) {
+        if constexpr (kGate) {
+          const __nv_bfloat16* gr = epi.gate + (size_t)min(row0 + lane, M - 1) * epi.ldc + col0;
+          if (col0 + 31 < N && (epi.ldc & 7) == 0) {
+#pragma unroll
+            for (int i = 0; i < 32; i += 8) {
+              const uint4 w = __ldg(reinterpret_cast<const uint4*>(gr + i));
+              const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&w);
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                v[i + 2 * u] = __low2float(h[u]) > 0.f ? v[i + 2 * u] * epi.alpha : 0.f;
+                v[i + 2 * u + 1] = __high2float(h[u]) > 0.f ? v[i + 2 * u + 1] * epi.alpha : 0.f;
+              }
+            }
+          } else {
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+              v[i] = col0 + i < N && __bfloat162float(gr[i]) > 0.f ? v[i] * epi.alpha : 0.f;
+          }
+        } else if (act) {
 #pragma unroll
           for (int i = 0; i < 32; ++i) {
             const int col = min(col0 + i, N - 1);
@@ -425,9 +445,13 @@ __global__ void __launch_bounds__(256) splitk_reduce(const float* __restrict__ p
       if (epi.kind == kEpiStoreF32) {
         epi.out_f32[(size_t)r * epi.ldc + c] = acc[i] * epi.alpha;
       } else {
-        z = acc[i] + (epi.bias ? epi.bias[c] : 0.f);
-        if (epi.act == kActRelu) z = fmaxf(z, 0.f);
-        else if (epi.act == kActSigmoid) z = sigmoidf(z);
+        if (epi.kind == kEpiReluGradBF16) {
+          z = __bfloat162float(epi.gate[(size_t)r * epi.ldc + c]) > 0.f ? acc[i] * epi.alpha : 0.f;
+        } else {
+          z = acc[i] + (epi.bias ? epi.bias[c] : 0.f);
+          if (epi.act == kActRelu) z = fmaxf(z, 0.f);
+          else if (epi.act == kActSigmoid) z = sigmoidf(z);
+        }
         const __nv_bfloat16 b = __float2bfloat16(z);
         if (epi.out_bf16) epi.out_bf16[(size_t)r * epi.ldc + c] = b;
         if (epi.out_f32) epi.out_f32[(size_t)r * epi.ldc + c] = z;
@@ -436,7 +460,7 @@ __global__ void __launch_bounds__(256) splitk_reduce(const float* __restrict__ p
     }
     tile[ty + 8 * i][tx] = z;
   }
-  if (epi.kind != kEpiBiasActBF16 || !epi.out_bf16_t) return;
+  if (epi.kind == kEpiStoreF32 || !epi.out_bf16_t) return;
   __syncthreads();
   // transposed: 16 rows of each of the 32 columns, lanes along the rows
   const int rr = threadIdx.x & 15, cq = threadIdx.x >> 4;  // 16 rows x 16 column pairs
@@ -502,8 +526,12 @@ cudaError_t gemm_device_setup(int* sms) {
   GemmDevice& d = g_gemm_dev[dev];
   bool& attr = BN == 256 ? d.attr256 : d.attr128;
   if (!attr) {
-    e = cudaFuncSetAttribute(gemm_bf16_tc<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(sizeof(GemmSmem<BN>) + 1024));
+    const int smem = (int)(sizeof(GemmSmem<BN>) + 1024);
+    e = cudaFuncSetAttribute(gemm_bf16_tc<BN, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             smem);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(gemm_bf16_tc<BN, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               smem);
     if (e != cudaSuccess) return e;
     attr = true;
   }
@@ -547,8 +575,9 @@ cudaError_t launch_bn(const CUtensorMap& ma, const CUtensorMap& mb, const GemmEp
   const long long items = tiles * splits;
   const int grid = (int)(items < sms ? items : sms);  // persistent: one CTA per SM
   float* part = splits > 1 ? ws : nullptr;
-  e = launch_pdl(gemm_bf16_tc<BN>, dim3((unsigned)grid), dim3(kGemmThreads), smem, st, ma, mb, epi,
-                 M, N, K, splits, kb_per, part, err);
+  const bool gate = !part && epi.kind == kEpiReluGradBF16;
+  e = launch_pdl(gate ? gemm_bf16_tc<BN, true> : gemm_bf16_tc<BN, false>, dim3((unsigned)grid),
+                 dim3(kGemmThreads), smem, st, ma, mb, epi, M, N, K, splits, kb_per, part, err);
   if (e != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess || splits == 1) return e;
   const dim3 rgrid((N + 31) / 32, (M + kRedRows - 1) / kRedRows);
   e = launch_pdl(splitk_reduce, rgrid, dim3(256), 0, st, (const float*)ws, splits, M, N, epi);

@@ -9,6 +9,7 @@ namespace synth {
 enum GemmEpiKind : int {
   kEpiStoreF32 = 0,     // out_f32[row][col] = alpha * acc
   kEpiBiasActBF16 = 1,  // z = act(acc + bias[col]) -> out_bf16 / out_bf16_t (transposed) / out_f32
+  kEpiReluGradBF16 = 2, // z = gate[row][col] > 0 ? alpha * acc : 0 -> as kEpiBiasActBF16
 };
 enum GemmAct : int { kActNone = 0, kActRelu = 1, kActSigmoid = 2 };
 
@@ -19,7 +20,8 @@ struct GemmEpilogue {
   __nv_bfloat16* out_bf16 = nullptr;
   __nv_bfloat16* out_bf16_t = nullptr;
   const float* bias = nullptr;
-  int ldc = 0;      // row stride (elements) of out_f32 / out_bf16
+  const __nv_bfloat16* gate = nullptr;  // the layer's activations, 16-byte aligned
+  int ldc = 0;      // row stride (elements) of out_f32 / out_bf16 / gate
   int ldc_t = 0;    // row stride of the transposed copy
   float alpha = 1.f;
 };

@@ -83,7 +83,8 @@ __global__ void transpose_bf16(const __nv_bfloat16* __restrict__ in, int rows, i
 __global__ void __launch_bounds__(256) mse_sigmoid_grad(
     const float* __restrict__ y, const float* __restrict__ target, int batch, int P, int P_pad,
     __nv_bfloat16* __restrict__ dz, __nv_bfloat16* __restrict__ dzt, float* __restrict__ dzf,
-    float* __restrict__ part, unsigned int* __restrict__ counter, float* __restrict__ loss) {
+    float* __restrict__ part, unsigned int* __restrict__ counter, float* __restrict__ loss,
+    float* __restrict__ loss_out) {
   pdl_wait();     // earlier kernels' writes are visible
   pdl_release();  // the next kernel may be scheduled
   __shared__ float red[8];
@@ -119,42 +120,8 @@ __global__ void __launch_bounds__(256) mse_sigmoid_grad(
   float t = 0.f;
   for (unsigned int k = 0; k < gridDim.x; ++k) t += reinterpret_cast<volatile float*>(part)[k];
   *counter = 0u;
-  if (loss) *loss = t / (float)(batch * P);
-}
-
-// Hidden layer: dZ = dH * relu'(Z) with relu'(Z) = (H > 0); writes dZ, dZ^T
-// and the FP32 dZ. A block covers 32 batch rows x 32 columns (32 x 8
-// threads); the transposed copy goes through shared memory so that its
-// stores are coalesced too.
-__global__ void __launch_bounds__(256) relu_grad(const float* __restrict__ dh,
-                                                 const __nv_bfloat16* __restrict__ h, int batch,
-                                                 int width, __nv_bfloat16* __restrict__ dz,
-                                                 __nv_bfloat16* __restrict__ dzt,
-                                                 float* __restrict__ dzf) {
-  pdl_wait();     // earlier kernels' writes are visible
-  pdl_release();  // the next kernel may be scheduled
-  __shared__ __nv_bfloat16 tile[32][34];
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const int c = blockIdx.x * 32 + tx, b0 = blockIdx.y * 32;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int b = b0 + ty + 8 * k;
-    __nv_bfloat16 gb = __float2bfloat16(0.f);
-    if (b < batch && c < width) {
-      const int64_t i = (int64_t)b * width + c;
-      const float g = __bfloat162float(h[i]) > 0.f ? dh[i] : 0.f;
-      gb = __float2bfloat16(g);
-      dz[i] = gb;
-      dzf[i] = g;
-    }
-    tile[ty + 8 * k][tx] = gb;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int cc = blockIdx.x * 32 + ty + 8 * k, b = b0 + tx;
-    if (cc < width && b < batch) dzt[(int64_t)cc * batch + b] = tile[tx][ty + 8 * k];
-  }
+  *loss = t / (float)(batch * P);
+  if (loss_out) *loss_out = *loss;
 }
 
 // Bias gradient: db[c] = sum_b dZ[b][c] from the FP32 dZ. A block covers 32
@@ -382,64 +349,105 @@ cudaError_t mlp_forward(const MlpLayout& L, char* base, const __nv_bfloat16* x, 
   return cudaGetLastError();
 }
 
-cudaError_t mlp_train_step(const MlpLayout& L, char* base, const __nv_bfloat16* x,
-                           const float* target, int batch, float lr, int step, float* loss_out,
-                           unsigned int* err, cudaStream_t st) {
+namespace {
+
+// The output gradients of a layer: bf16 [batch][ld], its transpose and FP32.
+struct LayerGrad {
+  __nv_bfloat16 *dz, *dzt;
+  float* dzf;
+};
+
+size_t grad_elems(const MlpLayout& L) {
+  return (size_t)L.max_batch * (L.dims[1] > L.out_pad ? L.dims[1] : L.out_pad);
+}
+
+// Layer 0 uses the layout's buffers; layers 1 to 3 the side memory.
+LayerGrad layer_grad(const MlpLayout& L, char* base, const MlpSide& side, int l) {
+  if (l == 0)
+    return {reinterpret_cast<__nv_bfloat16*>(base + L.dz),
+            reinterpret_cast<__nv_bfloat16*>(base + L.dzt), reinterpret_cast<float*>(base + L.dzf)};
+  const size_t n = grad_elems(L);
+  char* m = side.mem + (size_t)(l - 1) * 2 * al256(4 * n);
+  return {reinterpret_cast<__nv_bfloat16*>(m), reinterpret_cast<__nv_bfloat16*>(m + al256(2 * n)),
+          reinterpret_cast<float*>(m + al256(4 * n))};
+}
+
+}  // namespace
+
+cudaError_t mlp_side_create(const MlpLayout& L, MlpSide* s) {
+  cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&s->mem), 6 * al256(4 * grad_elems(L)));
+  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->st, cudaStreamNonBlocking);
+  cudaEvent_t* events[8] = {&s->begun, &s->h0t_ready, &s->gb0_ready, &s->done,
+                            &s->dz_ready[0], &s->dz_ready[1], &s->dz_ready[2], &s->dz_ready[3]};
+  for (cudaEvent_t* ev : events)
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
+  if (e != cudaSuccess) mlp_side_destroy(s);
+  return e;
+}
+
+void mlp_side_destroy(MlpSide* s) {
+  cudaEvent_t events[8] = {s->begun, s->h0t_ready, s->gb0_ready, s->done,
+                           s->dz_ready[0], s->dz_ready[1], s->dz_ready[2], s->dz_ready[3]};
+  for (cudaEvent_t ev : events)
+    if (ev) cudaEventDestroy(ev);
+  if (s->st) cudaStreamDestroy(s->st);
+  if (s->mem) cudaFree(s->mem);
+  *s = MlpSide{};
+}
+
+// The step's chain on st is what each kernel's inputs force: the forward, the
+// loss, each layer's input gradient with its ReLU, then layer 0's weight
+// gradient and Adam, which stream 1.5 GB. The rest -- the features'
+// transpose, bias gradients, the other layers' weight gradients and Adam, some
+// fifteen kernels of a few microseconds that fill a fraction of the GPU --
+// runs beside it on the model's own stream and has joined st when the step
+// returns to the caller's order. In one stream a step at batch 128 and 44160
+// inputs took 457 us, so 372.
+cudaError_t mlp_train_step(const MlpLayout& L, char* base, const MlpSide& side,
+                           const __nv_bfloat16* x, const float* target, int batch, float lr, int step,
+                           float* loss_out, unsigned int* err, cudaStream_t st) {
   if (batch % 8 != 0 || batch > L.max_batch) return cudaErrorInvalidValue;
-  cudaError_t e = mlp_forward(L, base, x, batch, true, nullptr, err, st);
-  if (e != cudaSuccess) return e;
+  cudaError_t e;
   __nv_bfloat16* h0t = reinterpret_cast<__nv_bfloat16*>(base + L.h0t);
+  if ((e = cudaEventRecord(side.begun, st)) != cudaSuccess ||
+      (e = cudaStreamWaitEvent(side.st, side.begun, 0)) != cudaSuccess)
+    return e;
   {
     dim3 g((L.dims[0] + 31) / 32, (batch + 31) / 32), b(32, 8);
-    if ((e = launch_pdl(transpose_bf16, g, b, 0, st, x, batch, L.dims[0], h0t)) != cudaSuccess)
+    if ((e = launch_pdl(transpose_bf16, g, b, 0, side.st, x, batch, L.dims[0], h0t)) != cudaSuccess ||
+        (e = cudaEventRecord(side.h0t_ready, side.st)) != cudaSuccess)
       return e;
   }
-  __nv_bfloat16* dz = reinterpret_cast<__nv_bfloat16*>(base + L.dz);
-  __nv_bfloat16* dzt = reinterpret_cast<__nv_bfloat16*>(base + L.dzt);
-  float* dh = reinterpret_cast<float*>(base + L.dh);
-  float* dzf = reinterpret_cast<float*>(base + L.dzf);
-  float* loss = reinterpret_cast<float*>(base + L.loss);
+  if ((e = mlp_forward(L, base, x, batch, true, nullptr, err, st)) != cudaSuccess) return e;
   const int P = L.dims[4], Pp = L.out_pad;
+  const LayerGrad out_grad = layer_grad(L, base, side, 3);
   if ((e = launch_pdl(mse_sigmoid_grad, dim3((batch * Pp + 255) / 256), dim3(256), 0, st,
-                      reinterpret_cast<const float*>(base + L.y), target, batch, P, Pp, dz, dzt,
-                      dzf, reinterpret_cast<float*>(base + L.loss_part),
-                      reinterpret_cast<unsigned int*>(base + L.loss_counter), loss)) != cudaSuccess)
+                      reinterpret_cast<const float*>(base + L.y), target, batch, P, Pp, out_grad.dz,
+                      out_grad.dzt, out_grad.dzf, reinterpret_cast<float*>(base + L.loss_part),
+                      reinterpret_cast<unsigned int*>(base + L.loss_counter),
+                      reinterpret_cast<float*>(base + L.loss), loss_out)) != cudaSuccess)
     return e;
-  for (int l = 3; l >= 0; --l) {
-    const int in = L.dims[l], out = L.dims[l + 1];
-    const int ldz = l == 3 ? Pp : out;
-    // bias and weight gradients: dW[out][in] = dZ^T[out][B] * H_{l}^T[in][B]^T
-    if ((e = launch_pdl(bias_grad, dim3((out + 31) / 32), dim3(256), 0, st, (const float*)dzf,
-                        batch, out, ldz, reinterpret_cast<float*>(base + L.gb[l]))) != cudaSuccess)
-      return e;
-    const __nv_bfloat16* hprev_t =
-        l == 0 ? h0t : reinterpret_cast<const __nv_bfloat16*>(base + L.ht[l]);
+  // bias and weight gradients of layer l: dW[out][in] = dZ^T[out][B] * H_l^T[in][B]^T
+  auto bias_gradient = [&](int l) {
+    const int out = L.dims[l + 1];
+    return launch_pdl(bias_grad, dim3((out + 31) / 32), dim3(256), 0, side.st,
+                      (const float*)layer_grad(L, base, side, l).dzf, batch, out, l == 3 ? Pp : out,
+                      reinterpret_cast<float*>(base + L.gb[l]));
+  };
+  auto weight_gradient = [&](int l, cudaStream_t on) {
     GemmEpilogue ew;
     ew.kind = kEpiStoreF32;
     ew.out_f32 = reinterpret_cast<float*>(base + L.gw[l]);
-    ew.ldc = in;
-    if ((e = gemm_bf16(dzt, batch, hprev_t, batch, out, in, batch, ew, err, st)) != cudaSuccess)
-      return e;
-    if (l > 0) {
-      // dH_{l}[B][in] = dZ[B][ldz] * W^T[in][ldz]^T
-      GemmEpilogue eh;
-      eh.kind = kEpiStoreF32;
-      eh.out_f32 = dh;
-      eh.ldc = in;
-      if ((e = gemm_bf16(dz, ldz, reinterpret_cast<const __nv_bfloat16*>(base + L.wt[l]), ldz,
-                         batch, in, ldz, eh, err, st, reinterpret_cast<float*>(base + L.splitk),
-                         L.splitk_bytes)) != cudaSuccess)
-        return e;
-      if ((e = launch_pdl(relu_grad, dim3((in + 31) / 32, (batch + 31) / 32), dim3(256), 0, st,
-                          (const float*)dh, reinterpret_cast<const __nv_bfloat16*>(base + L.h[l]),
-                          batch, in, dz, dzt, dzf)) != cudaSuccess)
-        return e;
-    }
-  }
-  // Adam: each layer's weights and bias in one launch
+    ew.ldc = L.dims[l];
+    const __nv_bfloat16* hprev_t =
+        l == 0 ? h0t : reinterpret_cast<const __nv_bfloat16*>(base + L.ht[l]);
+    return gemm_bf16(layer_grad(L, base, side, l).dzt, batch, hprev_t, batch, L.dims[l + 1],
+                     L.dims[l], batch, ew, err, on);
+  };
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
   const float c1 = 1.f - powf(b1, (float)step), c2 = 1.f - powf(b2, (float)step);
-  for (int l = 0; l < 4; ++l) {
+  // Adam: a layer's weights and bias in one launch
+  auto adam = [&](int l, cudaStream_t on) {
     const int in = L.dims[l], out = L.dims[l + 1];
     float* w = reinterpret_cast<float*>(base + L.w[l]);
     const float* g = reinterpret_cast<const float*>(base + L.gw[l]);
@@ -453,23 +461,50 @@ cudaError_t mlp_train_step(const MlpLayout& L, char* base, const __nv_bfloat16* 
     if (l == 0) {
       // no transposed copy: a vectorised stream (in * out is a multiple of 4)
       const int64_t n4 = (int64_t)in * out / 4;
-      if ((e = launch_pdl(adam_update_vec4, dim3(grid_of(n4 + out)), dim3(256), 0, st,
-                          reinterpret_cast<float4*>(w), reinterpret_cast<const float4*>(g),
-                          reinterpret_cast<float4*>(mw), reinterpret_cast<float4*>(vw), n4, lr, b1,
-                          b2, eps, c1, c2, reinterpret_cast<uint2*>(wb), bias)) != cudaSuccess)
-        return e;
-    } else {
-      const int outp = l == 3 ? Pp : out;
-      if ((e = launch_pdl(adam_update_tiled, dim3((in + 31) / 32, (out + 31) / 32), dim3(256), 0,
-                          st, w, g, mw, vw, out, in, lr, b1, b2, eps, c1, c2, wb,
-                          reinterpret_cast<__nv_bfloat16*>(base + L.wt[l]), outp, bias)) !=
-          cudaSuccess)
-        return e;
+      return launch_pdl(adam_update_vec4, dim3(grid_of(n4 + out)), dim3(256), 0, on,
+                        reinterpret_cast<float4*>(w), reinterpret_cast<const float4*>(g),
+                        reinterpret_cast<float4*>(mw), reinterpret_cast<float4*>(vw), n4, lr, b1, b2,
+                        eps, c1, c2, reinterpret_cast<uint2*>(wb), bias);
     }
+    return launch_pdl(adam_update_tiled, dim3((in + 31) / 32, (out + 31) / 32), dim3(256), 0, on, w,
+                      g, mw, vw, out, in, lr, b1, b2, eps, c1, c2, wb,
+                      reinterpret_cast<__nv_bfloat16*>(base + L.wt[l]), l == 3 ? Pp : out, bias);
+  };
+  for (int l = 3; l >= 0; --l) {
+    // layer l's output gradients are there; in this order the side stream has
+    // also seen every product that reads a weight copy Adam rewrites
+    if ((e = cudaEventRecord(side.dz_ready[l], st)) != cudaSuccess ||
+        (e = cudaStreamWaitEvent(side.st, side.dz_ready[l], 0)) != cudaSuccess ||
+        (e = bias_gradient(l)) != cudaSuccess)
+      return e;
+    if (l == 0) break;
+    if ((e = weight_gradient(l, side.st)) != cudaSuccess) return e;
+    // dH_l[B][in] = dZ_l[B][ldz] * W_l^T[in][ldz]^T, through the ReLU of layer l - 1
+    const int in = L.dims[l], ldz = l == 3 ? Pp : L.dims[l + 1];
+    const LayerGrad below = layer_grad(L, base, side, l - 1);
+    GemmEpilogue eh;
+    eh.kind = kEpiReluGradBF16;
+    eh.gate = reinterpret_cast<const __nv_bfloat16*>(base + L.h[l]);
+    eh.out_bf16 = below.dz;
+    eh.out_bf16_t = below.dzt;
+    eh.out_f32 = below.dzf;
+    eh.ldc = in;
+    eh.ldc_t = batch;
+    if ((e = gemm_bf16(layer_grad(L, base, side, l).dz, ldz,
+                       reinterpret_cast<const __nv_bfloat16*>(base + L.wt[l]), ldz, batch, in, ldz,
+                       eh, err, st, reinterpret_cast<float*>(base + L.splitk), L.splitk_bytes)) !=
+        cudaSuccess)
+      return e;
   }
-  // the loss last, so that no copy splits the chain of kernels above
-  if (loss_out &&
-      (e = cudaMemcpyAsync(loss_out, loss, sizeof(float), cudaMemcpyDeviceToDevice, st)) != cudaSuccess)
+  if ((e = cudaEventRecord(side.gb0_ready, side.st)) != cudaSuccess) return e;
+  for (int l = 3; l >= 1; --l)
+    if ((e = adam(l, side.st)) != cudaSuccess) return e;
+  if ((e = cudaEventRecord(side.done, side.st)) != cudaSuccess ||
+      (e = cudaStreamWaitEvent(st, side.h0t_ready, 0)) != cudaSuccess ||
+      (e = weight_gradient(0, st)) != cudaSuccess ||
+      (e = cudaStreamWaitEvent(st, side.gb0_ready, 0)) != cudaSuccess ||
+      (e = adam(0, st)) != cudaSuccess ||
+      (e = cudaStreamWaitEvent(st, side.done, 0)) != cudaSuccess)
     return e;
   return cudaGetLastError();
 }

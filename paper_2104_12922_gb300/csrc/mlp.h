@@ -21,15 +21,28 @@ struct MlpLayout {
   size_t total;
 };
 
+// What a training step runs beside its main chain on: a stream of the model's
+// own with the events that order the two, and per-layer output gradients, so
+// that a layer's weight gradient can read its own while the chain makes the
+// next layer's. Not part of the saved layout.
+struct MlpSide {
+  cudaStream_t st = nullptr;
+  cudaEvent_t begun = nullptr, h0t_ready = nullptr, gb0_ready = nullptr, done = nullptr;
+  cudaEvent_t dz_ready[4] = {};
+  char* mem = nullptr;
+};
+cudaError_t mlp_side_create(const MlpLayout& L, MlpSide* s);
+void mlp_side_destroy(MlpSide* s);
+
 MlpLayout mlp_layout(int in_dim, int hidden, int out_dim, int max_batch, size_t splitk_bytes);
 cudaError_t mlp_init(const MlpLayout& L, char* base, uint64_t seed, cudaStream_t st);
 // y_out [batch][out] (FP32 sigmoid outputs), or the model's own buffer if NULL.
 cudaError_t mlp_forward(const MlpLayout& L, char* base, const __nv_bfloat16* x, int batch,
                         bool keep_transposes, float* y_out, unsigned int* err, cudaStream_t st);
 // Forward, MSE against target [batch][out], backward, one Adam step (step >= 1).
-cudaError_t mlp_train_step(const MlpLayout& L, char* base, const __nv_bfloat16* x,
-                           const float* target, int batch, float lr, int step, float* loss_out,
-                           unsigned int* err, cudaStream_t st);
+cudaError_t mlp_train_step(const MlpLayout& L, char* base, const MlpSide& side,
+                           const __nv_bfloat16* x, const float* target, int batch, float lr, int step,
+                           float* loss_out, unsigned int* err, cudaStream_t st);
 // Hidden activations H_layer (layer 1..3, bf16, of the last forward or
 // training step) as FP32 [batch][hidden].
 cudaError_t mlp_hidden_f32(const MlpLayout& L, const char* base, int layer, int batch, float* dst,

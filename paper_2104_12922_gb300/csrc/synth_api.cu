@@ -423,6 +423,7 @@ synth_status synth_param_adam(synth_handle h, float* u_dev, const float* grad_de
 struct synth_model_s {
   synth_handle synth = nullptr;
   MlpLayout L;
+  MlpSide side;
   char* mem = nullptr;        // MlpLayout tensors
   void* work = nullptr;       // audio, params, features, log-mel workspace
   float* audio = nullptr;     // [max_batch][N]
@@ -458,8 +459,10 @@ synth_status synth_model_create(synth_handle h, int32_t max_batch, uint64_t seed
     delete m;
     return SYNTH_ERR_OOM;
   }
-  if (cudaMalloc(&m->work, a_bytes + p_bytes + f_bytes + mel_bytes) != cudaSuccess) {
+  if (cudaMalloc(&m->work, a_bytes + p_bytes + f_bytes + mel_bytes) != cudaSuccess ||
+      mlp_side_create(m->L, &m->side) != cudaSuccess) {
     cudaFree(m->mem);
+    cudaFree(m->work);
     delete m;
     return SYNTH_ERR_OOM;
   }
@@ -471,6 +474,7 @@ synth_status synth_model_create(synth_handle h, int32_t max_batch, uint64_t seed
   if (mlp_init(m->L, m->mem, seed, 0) != cudaSuccess ||
       logmel_fft_init(h->vc.sample_rate, m->mel_ws, 0) != cudaSuccess ||
       cudaDeviceSynchronize() != cudaSuccess) {
+    mlp_side_destroy(&m->side);
     cudaFree(m->mem);
     cudaFree(m->work);
     delete m;
@@ -482,6 +486,7 @@ synth_status synth_model_create(synth_handle h, int32_t max_batch, uint64_t seed
 
 synth_status synth_model_destroy(synth_model m) {
   if (!m) return SYNTH_ERR_ARG;
+  mlp_side_destroy(&m->side);
   cudaFree(m->mem);
   cudaFree(m->work);
   delete m;
@@ -549,8 +554,8 @@ synth_status synth_model_train_features(synth_model m, const void* features_dev,
   ScratchHeader* hdr = static_cast<ScratchHeader*>(m->synth->scratch);
   m->step += 1;
   m->last_batch = batch;
-  return check_cuda(mlp_train_step(m->L, m->mem, static_cast<const __nv_bfloat16*>(features_dev),
-                                   target_dev, batch, lr, m->step, loss_dev, &hdr->error,
+  return check_cuda(mlp_train_step(m->L, m->mem, m->side,
+                                   static_cast<const __nv_bfloat16*>(features_dev), target_dev, batch, lr, m->step, loss_dev, &hdr->error,
                                    static_cast<cudaStream_t>(stream)));
 }
 
