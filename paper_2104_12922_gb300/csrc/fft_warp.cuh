@@ -44,45 +44,13 @@ __host__ __device__ constexpr int bitrev(int r) {
 }
 
 // In-register radix-2 decimation-in-frequency L-point DFT (L = 8, 16, 32) of
-// re/im[O .. O + L): X[k] = sum_n x[n] e^(-2 pi i n k / L) for natural-order
-// input, X[k] left in register O + bitrev<L>(k). The twiddle of a butterfly
-// of half-width h at offset j is e^(-2 pi i j / (2h)) = W32^(16 j / h); the
-// trivial ones (1 and -i) cost no multiplications.
-template <int L, int O>
-__device__ __forceinline__ void dft(float (&re)[32], float (&im)[32]) {
-#pragma unroll
-  for (int half = L / 2; half >= 1; half >>= 1) {
-#pragma unroll
-    for (int g = 0; g < L; g += 2 * half) {
-#pragma unroll
-      for (int j = 0; j < half; ++j) {
-        const int p = O + g + j, q = O + g + j + half;
-        const float ur = re[p], ui = im[p], vr = re[q], vi = im[q];
-        re[p] = ur + vr;
-        im[p] = ui + vi;
-        const float dr = ur - vr, di = ui - vi;
-        const int tw = j * (16 / half);
-        if (tw == 0) {
-          re[q] = dr;
-          im[q] = di;
-        } else if (tw == 8) {  // -i
-          re[q] = di;
-          im[q] = -dr;
-        } else {
-          const float wr = w32_re(tw), wi = w32_im(tw);
-          re[q] = fmaf(dr, wr, -di * wi);
-          im[q] = fmaf(dr, wi, di * wr);
-        }
-      }
-    }
-  }
-}
-
-// The same transform of complex values held as (re, im) pairs: the butterflies'
-// sums and differences are packed instructions, the twiddles scalar ones on
-// the halves (a packed constant would take a register pair of its own). The
-// results are those of the scalar form, bit for bit. 32 points: 326
-// instructions instead of 456.
+// z[O .. O + L), each a (re, im) pair: X[k] = sum_n x[n] e^(-2 pi i n k / L) for
+// natural-order input, X[k] left in register O + bitrev<L>(k). The twiddle of
+// a butterfly of half-width h at offset j is e^(-2 pi i j / (2h)) = W32^(16 j / h);
+// the trivial ones (1 and -i) cost no multiplications. The butterflies' sums
+// and differences are packed instructions, the twiddles scalar ones on the
+// halves (a packed constant would take a register pair of its own): 326
+// instructions for 32 points, 456 with scalar butterflies, the same results.
 template <int L, int O>
 __device__ __forceinline__ void dft(f32x2 (&z)[32]) {
 #pragma unroll
@@ -115,12 +83,12 @@ __device__ __forceinline__ void dft(f32x2 (&z)[32]) {
 // The R-point DFTs of all 32 / R frames a lane holds (frame f in registers
 // f R .. f R + R - 1).
 template <int R>
-__device__ __forceinline__ void dft_frames(float (&re)[32], float (&im)[32]) {
-  dft<R, 0>(re, im);
-  if constexpr (R <= 16) dft<R, R>(re, im);
+__device__ __forceinline__ void dft_frames(f32x2 (&z)[32]) {
+  dft<R, 0>(z);
+  if constexpr (R <= 16) dft<R, R>(z);
   if constexpr (R <= 8) {
-    dft<R, 2 * R>(re, im);
-    dft<R, 3 * R>(re, im);
+    dft<R, 2 * R>(z);
+    dft<R, 3 * R>(z);
   }
 }
 

@@ -175,21 +175,20 @@ __global__ void __launch_bounds__(kThreadsMr, 2)
     // one pass per warp: frames lf0 .. lf0 + FPW - 1 of the item
     const int lf0 = warp * C::FPW;
     float re[32], im[32];
+    f32x2 z[32];
     if (lf0 < Gi) {
       // ---- forward: z[32 a + lane] of frames lf0 .. lf0 + FPW - 1, windowed
 #pragma unroll
       for (int fr = 0; fr < C::FPW; ++fr) {
         const int lf = min(lf0 + fr, Gi - 1);
-        const float2* s2 = reinterpret_cast<const float2*>(sg + lf * C::hop);
+        const f32x2* s2 = reinterpret_cast<const f32x2*>(sg + lf * C::hop);
+        const f32x2* w2 = reinterpret_cast<const f32x2*>(S.win);
 #pragma unroll
-        for (int a = 0; a < R; ++a) {
-          const float2 sv = s2[32 * a + lane];
-          const float2 wv = S.win[32 * a + lane];
-          re[fr * R + a] = sv.x * wv.x;
-          im[fr * R + a] = sv.y * wv.y;
-        }
+        for (int a = 0; a < R; ++a) z[fr * R + a] = mul2(s2[32 * a + lane], w2[32 * a + lane]);
       }
-      fftw::dft_frames<R>(re, im);
+      fftw::dft_frames<R>(z);
+#pragma unroll
+      for (int i = 0; i < 32; ++i) unpack2(z[i], re[i], im[i]);
 #pragma unroll
       for (int fr = 0; fr < C::FPW; ++fr)
 #pragma unroll
@@ -216,7 +215,7 @@ __global__ void __launch_bounds__(kThreadsMr, 2)
         for (int r = 0; r < R; ++r) B[(fr * R + bitrev<R>(r)) * kLdMr + lane] = im[fr * R + r];
       __syncwarp();
 #pragma unroll
-      for (int b = 0; b < 32; ++b) im[b] = B[lane * kLdMr + b];
+      for (int b = 0; b < 32; ++b) z[b] = pack2(re[b], B[lane * kLdMr + b]);
       __syncwarp();
       // the target rows of this warp's frames into B (free until the inverse
       // transposes) by one bulk copy, in flight during the 32-point DFTs
@@ -227,7 +226,9 @@ __global__ void __launch_bounds__(kThreadsMr, 2)
         mbar::expect_tx(&S.mbar[warp], bytes);
         mbar::bulk_g2s(B, logy + ((size_t)v * F + f0 + lf0) * C::ldl, bytes, &S.mbar[warp]);
       }
-      fftw::dft<32, 0>(re, im);  // Z[k1 + R k2] of frame phi in register bitrev<32>(k2)
+      fftw::dft<32, 0>(z);  // Z[k1 + R k2] of frame phi in register bitrev<32>(k2)
+#pragma unroll
+      for (int i = 0; i < 32; ++i) unpack2(z[i], re[i], im[i]);
       if (mode != kMrTarget) {
         if (!mbar::wait(&S.mbar[warp], mb_phase, kMrWaitLimit) && lane == 0) atomicOr(err, 1u);
         mb_phase ^= 1;
@@ -339,17 +340,14 @@ __global__ void __launch_bounds__(kThreadsMr, 2)
       // 32-point inverse DFT over k2 (the swap of real and imaginary parts
       // turns the forward transform into the inverse one)
       {
-        float tr[32], ti[32];
 #pragma unroll
-        for (int k2 = 0; k2 < 32; ++k2) {
-          tr[k2] = re[bitrev<32>(k2)];
-          ti[k2] = im[bitrev<32>(k2)];
-        }
-        fftw::dft<32, 0>(ti, tr);  // T[b] in register bitrev<32>(b)
+        for (int k2 = 0; k2 < 32; ++k2) z[k2] = pack2(im[bitrev<32>(k2)], re[bitrev<32>(k2)]);
+        fftw::dft<32, 0>(z);  // T[b] in register bitrev<32>(b)
 #pragma unroll
         for (int r = 0; r < 32; ++r) {
           const int b = bitrev<32>(r);
-          float yr = tr[r], yi = ti[r];
+          float yr, yi;
+          unpack2(z[r], yi, yr);
           if (b != 0 && k1 != 0) {
             const float2 w = S.twi[b * R + k1];
             const float t0 = fmaf(yr, w.x, -yi * w.y);
@@ -375,21 +373,25 @@ __global__ void __launch_bounds__(kThreadsMr, 2)
 #pragma unroll
       for (int fr = 0; fr < C::FPW; ++fr)
 #pragma unroll
-        for (int q = 0; q < R; ++q) im[fr * R + q] = B[(fr * R + q) * kLdMr + lane];
+        for (int q = 0; q < R; ++q)
+          z[fr * R + q] = pack2(B[(fr * R + q) * kLdMr + lane], re[fr * R + q]);
       __syncwarp();
-      fftw::dft_frames<R>(im, re);  // z[32 a + lane] of frame fr in register fr R + bitrev<R>(a)
+      fftw::dft_frames<R>(z);  // z[32 a + lane] of frame fr in register fr R + bitrev<R>(a)
+#pragma unroll
+      for (int i = 0; i < 32; ++i) unpack2(z[i], im[i], re[i]);
       }
     }
     if (mode == kMrLossGrad) {
       // the item's frame gradients (times the window) summed into its padded
       // segment, over the audio it no longer needs; frames four hops apart do
       // not overlap, so the four residue classes of the frame index add in
-      // turn (a fixed order: the sums are deterministic)
+      // turn (a fixed order: the sums are deterministic; one copy of the code, the
+      // kernel is short of instruction cache)
       __syncthreads();
       for (int j = 4 * threadIdx.x; j < len; j += 4 * kThreadsMr)
         *reinterpret_cast<float4*>(sg + j) = make_float4(0.f, 0.f, 0.f, 0.f);
       __syncthreads();
-#pragma unroll
+#pragma unroll 1
       for (int c = 0; c < 4; ++c) {
 #pragma unroll
         for (int fr = 0; fr < C::FPW; ++fr) {
