@@ -121,10 +121,13 @@ __device__ __forceinline__ void stage_segment(float* dst, const float* __restric
   asm volatile("cp.async.commit_group;\n" ::: "memory");
 }
 
-template <int R>
+// The pass is a template argument: with it as a run-time one, the unrolled code
+// of every bin held all three passes, 155 KB where an SM's instruction cache
+// holds 128, and instruction fetch led the stalls.
+template <int R, int mode>
 __global__ void __launch_bounds__(kThreadsMr, 2)
     mr_fft_kernel(const float* __restrict__ sig, int N, int F, int batch, MrTables t, float eps,
-                  float scale, int mode, float* __restrict__ logy, double* __restrict__ loss_item,
+                  float scale, float* __restrict__ logy, double* __restrict__ loss_item,
                   float* __restrict__ part, unsigned int* __restrict__ err) {
   using C = MrCfg<R>;
   extern __shared__ __align__(16) unsigned char mr_raw[];
@@ -549,33 +552,38 @@ cudaError_t mr_tables_fill(int R, void* dst, cudaStream_t st) {
 
 int r_of(int n_fft) { return n_fft == 512 ? 8 : n_fft == 1024 ? 16 : n_fft == 2048 ? 32 : 0; }
 
-template <int R>
+template <int R, int mode>
 cudaError_t mr_launch(const float* sig, int N, int F, int batch, const char* tables, float eps,
-                      float scale, int mode, float* logy, double* loss_item, float* part,
-                      unsigned int* err, cudaStream_t st) {
+                      float scale, float* logy, double* loss_item, float* part, unsigned int* err,
+                      cudaStream_t st) {
   const int smem = (int)sizeof(MrSmem<R>);
   int grid_cap = 0;  // resident CTAs on the current device
-  const cudaError_t ge =
-      resident_grid(reinterpret_cast<const void*>(mr_fft_kernel<R>), kThreadsMr, smem, &grid_cap);
+  const cudaError_t ge = resident_grid(reinterpret_cast<const void*>(mr_fft_kernel<R, mode>),
+                                       kThreadsMr, smem, &grid_cap);
   if (ge != cudaSuccess) return ge;
   const int64_t items = (int64_t)((F + MrCfg<R>::G - 1) / MrCfg<R>::G) * batch;
   if (items >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
   const int grid = (int)std::min<int64_t>(items, grid_cap);
-  mr_fft_kernel<R><<<grid, kThreadsMr, smem, st>>>(sig, N, F, batch, mr_tables(R, tables), eps,
-                                                   scale, mode, logy, loss_item, part, err);
+  mr_fft_kernel<R, mode><<<grid, kThreadsMr, smem, st>>>(sig, N, F, batch, mr_tables(R, tables), eps,
+                                                         scale, logy, loss_item, part, err);
   return cudaGetLastError();
 }
 
 cudaError_t mr_pass(int n_fft, const float* sig, int N, int F, int batch, const char* tables,
                     float eps, float scale, int mode, float* logy, double* loss_item, float* part,
                     unsigned int* err, cudaStream_t st) {
-#define SYNTH_MR_ARGS sig, N, F, batch, tables, eps, scale, mode, logy, loss_item, part, err, st
+#define SYNTH_MR_ARGS sig, N, F, batch, tables, eps, scale, logy, loss_item, part, err, st
+#define SYNTH_MR_PASS(R)                                                  \
+  return mode == kMrTarget ? mr_launch<R, kMrTarget>(SYNTH_MR_ARGS)       \
+         : mode == kMrLoss ? mr_launch<R, kMrLoss>(SYNTH_MR_ARGS)         \
+                           : mr_launch<R, kMrLossGrad>(SYNTH_MR_ARGS)
   switch (r_of(n_fft)) {
-    case 8: return mr_launch<8>(SYNTH_MR_ARGS);
-    case 16: return mr_launch<16>(SYNTH_MR_ARGS);
-    case 32: return mr_launch<32>(SYNTH_MR_ARGS);
+    case 8: SYNTH_MR_PASS(8);
+    case 16: SYNTH_MR_PASS(16);
+    case 32: SYNTH_MR_PASS(32);
     default: return cudaErrorInvalidValue;
   }
+#undef SYNTH_MR_PASS
 #undef SYNTH_MR_ARGS
 }
 
