@@ -1,6 +1,5 @@
 // control_pipeline.cuh -- the control-rate part of the Voice as separate
-// module kernels over device buffers (used by the plain render and by the
-// adjoint's forward recomputation).
+// module kernels over device buffers (the plain render's).
 #pragma once
 
 #include "control_ff.cuh"
@@ -30,10 +29,4 @@ ControlBuffers control_carve(const VoiceConst& vc, int batch, void* ws);
 void launch_control_pipeline(const VoiceConst& vc, uint64_t seed, uint64_t batch_index, int batch,
                              const float* params_in, float* params_out, const ControlBuffers& cb,
                              cudaStream_t st);
-// The same buffers, bit for bit, from one kernel (one CTA per voice, the
-// steps separated by barriers); hdr takes the bounds-checked build's errors.
-void launch_control_fused(const VoiceConst& vc, uint64_t seed, uint64_t batch_index, int batch,
-                          const float* params_in, float* params_out, const ControlBuffers& cb,
-                          ScratchHeader* hdr, cudaStream_t st);
-
 }  // namespace synth

@@ -6,29 +6,38 @@
 // Where the forward takes a branch (envelope section, clamp, Nyquist cap,
 // square LFO) the derivative is that of the branch taken.
 //
-// Passes (all on the caller's stream, buffers in the caller's workspace):
-//  1. forward recomputation of the control rate (control_pipeline.cuh: the
-//     plain form's module steps in one kernel, one CTA per voice); its
+// Three kernels (all on the caller's stream, buffers in the caller's workspace):
+//  1. bwd_recompute: the forward control rate, one CTA per voice, in the fused
+//     render's arithmetic (float-float chain, fixed-point phase sums); its
 //     per-interval phase descriptions are the checkpoints from which the
 //     audio-rate values are rebuilt;
-//  2. audio-rate reverse pass, one warp per control interval: rebuilds every
-//     sample, forms d/d(phase) of both VCOs, the amplitude, drive, shape and
-//     mixer-gain partials, and the interval's moments for the reverse phase
-//     scan (see bwd_samples);
-//  3. reverse scan over intervals (FP64): with C_k = sum of d/d(phase) over
-//     all samples from interval k on, the pitch adjoint of control point k is
-//     (ln 2 / 12) (M1_k + F1_k C_{k+1} + M2_{k-1} + F2_{k-1} C_k);
-//  4. control-rate reverse sweep per voice: modulation mixer, LFOs (with a
-//     reverse scan of the LFO phase adjoint), ADSRs, range map -> d/du.
+//  2. bwd_samples: audio-rate reverse pass, eight lanes per control interval:
+//     rebuilds every sample, forms d/d(phase) of both VCOs, the amplitude,
+//     drive, shape and mixer-gain partials, and the interval's moments for the
+//     reverse phase scan;
+//  3. bwd_control, one CTA per voice: the reverse scan over intervals (FP64):
+//     with C_k = sum of d/d(phase) over all samples from interval k on, the
+//     pitch adjoint of control point k is
+//     (ln 2 / 12) (M1_k + F1_k C_{k+1} + M2_{k-1} + F2_{k-1} C_k); then the
+//     control-rate reverse sweep: modulation mixer, LFOs (with a reverse scan of
+//     the LFO phase adjoint), ADSRs, range map -> d/du.
+//
+// What bounds it: at 64 voices of 1 s the 11 MB of audio gradient take 2 us; the
+// per-voice kernels are latency on 64 of 152 SMs, the sample pass is
+// instruction issue. So a step goes over the (envelope, point), (LFO, point) or
+// (VCO, interval) pairs of a voice and not over points alone, phase sums are
+// integers (an FP64 scan waits on the narrow FP64 pipe), and an interval's 21
+// sums are added up over 8 lanes, not 32. Kernels of the plain form's modules,
+// a warp per interval and a scan kernel that handed FP64 point adjoints on took
+// 110.6 us; now 79.2 us (the three under a profiler: 20, 33 and 30).
 
-#include "control_pipeline.cuh"
+#include "control_ff.cuh"
 #include "internal.h"
 
 namespace synth {
 
 namespace {
 
-constexpr int kBT = 256;
 constexpr int kStat = 21;  // per-interval partial sums written by bwd_samples
 // stat layout: [0..4] sine T, M1, F1, M2, F2; [5..9] square-saw T, M1, F1, M2, F2;
 // [10..12] amp grads to the left point (sine, sq, noise); [13..15] to the right
@@ -36,22 +45,40 @@ constexpr int kStat = 21;  // per-interval partial sums written by bwd_samples
 
 size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
 
-struct BwdLayout {
-  size_t stat, gpt, vacc, dtheta, denv, total;
+struct AdjBuffers {
+  float* y;       // [B][80] human-range parameters (78 used)
+  float* mix;     // [B][4] mixer gains (3), square-saw shape
+  float* env;     // [B][6][P] ADSRs at the control points
+  float* phase;   // [B][2][P] LFO phases (cycles, wrapped)
+  float* dest;    // [B][5][P] modulation mixer outputs
+  SegVco* seg;    // [B][2][K] VCO interval descriptions
+  float* kappa;   // [B][2][K] square-saw drive and 1/tanh(drive)
+  float* stat;    // [B][K][kStat]
+  double2* csum;  // [B][K] both VCOs' sums of d/d(phase) over all later intervals
+  float* dtheta;  // [B][2][P]
+  float* denv;    // [B][6][P]
+  size_t total;
 };
 
-BwdLayout bwd_layout(const VoiceConst& vc, int B, size_t base) {
-  const size_t P = (size_t)vc.K + 1, K = (size_t)vc.K;
-  BwdLayout L;
-  size_t o = base;
-  auto take = [&](size_t bytes) { size_t at = o; o = al256(o + bytes); return at; };
-  L.stat = take(sizeof(float) * B * K * kStat);
-  L.gpt = take(sizeof(double) * 2 * B * P * 5);
-  L.vacc = take(sizeof(double) * B * 8);
-  L.dtheta = take(sizeof(float) * B * 2 * P);
-  L.denv = take(sizeof(float) * B * 6 * P);
-  L.total = o;
-  return L;
+AdjBuffers adj_carve(const VoiceConst& vc, int batch, void* ws) {
+  const size_t B = (size_t)batch, P = (size_t)vc.K + 1, K = (size_t)vc.K;
+  char* base = static_cast<char*>(ws);
+  size_t o = 0;
+  auto take = [&](size_t bytes) { char* at = base ? base + o : nullptr; o += al256(bytes); return at; };
+  AdjBuffers b;
+  b.y = reinterpret_cast<float*>(take(sizeof(float) * B * 80));
+  b.mix = reinterpret_cast<float*>(take(sizeof(float) * B * 4));
+  b.env = reinterpret_cast<float*>(take(sizeof(float) * B * 6 * P));
+  b.phase = reinterpret_cast<float*>(take(sizeof(float) * B * 2 * P));
+  b.dest = reinterpret_cast<float*>(take(sizeof(float) * B * 5 * P));
+  b.seg = reinterpret_cast<SegVco*>(take(sizeof(SegVco) * B * 2 * K));
+  b.kappa = reinterpret_cast<float*>(take(sizeof(float) * B * 2 * K));
+  b.stat = reinterpret_cast<float*>(take(sizeof(float) * B * K * kStat));
+  b.csum = reinterpret_cast<double2*>(take(sizeof(double2) * B * K));
+  b.dtheta = reinterpret_cast<float*>(take(sizeof(float) * B * 2 * P));
+  b.denv = reinterpret_cast<float*>(take(sizeof(float) * B * 6 * P));
+  b.total = o;
+  return b;
 }
 
 __device__ __forceinline__ float warp_sum(float v) {
@@ -66,252 +93,328 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 }
 
 // ---------------------------------------------------------------------------
-// 2. audio-rate reverse pass. Warp w of a block takes control interval k; lane
-// l takes samples 4l..4l+3 of it (R <= 128). Four blocks per SM (64
-// registers, a small spill) run it faster than three with no spill.
+// 1. forward control rate of a voice, kCP control points (kCP - 1 intervals) at
+// a time. Threads 0 .. kCP - 1 take the first LFO and VCO, the others the second.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kBT, 4) bwd_samples(const __grid_constant__ VoiceConst vc,
+constexpr int kCT = 1024;
+constexpr int kCP = kCT / 2;
+constexpr int kCW = kCP / 32;  // warps of a half
+
+struct RecomputeSmem {
+  FFTables T;
+  VoiceFF V;
+  ff y[kNumParams];
+  // the six envelopes; an LFO's output then takes the place of its amplitude
+  // envelope (3, 5), a VCO's pitch that of an LFO's rate envelope (2, 4)
+  ff env[6][kCP];
+  unsigned long long p0[4];  // initial phases: LFOs, VCOs
+  unsigned long long warp_tot[2][kCW];
+};
+
+// Exclusive sum over each half of the block; tot: the half's whole sum.
+__device__ __forceinline__ unsigned long long half_scan(RecomputeSmem& s, unsigned long long x,
+                                                        unsigned long long& tot) {
+  const int lane = threadIdx.x & 31, half = threadIdx.x / kCP, warp = (threadIdx.x % kCP) >> 5;
+  unsigned long long in = x;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long n = __shfl_up_sync(0xffffffffu, in, o);
+    if (lane >= o) in += n;
+  }
+  __syncthreads();  // the earlier scan's totals are read
+  if (lane == 31) s.warp_tot[half][warp] = in;
+  __syncthreads();
+  unsigned long long before = 0;
+  tot = 0;
+#pragma unroll
+  for (int w = 0; w < kCW; ++w) {
+    const unsigned long long t = s.warp_tot[half][w];
+    if (w < warp) before += t;
+    tot += t;
+  }
+  return before + in - x;
+}
+
+__global__ void __launch_bounds__(kCT) bwd_recompute(const __grid_constant__ VoiceConst vc, int batch,
+                                                     const float* __restrict__ params,
+                                                     const AdjBuffers b, ScratchHeader* hdr) {
+  __shared__ RecomputeSmem s;
+  const int v = blockIdx.x, tid = threadIdx.x, half = tid / kCP, p = tid % kCP;
+  const int K = vc.K, P = K + 1;
+  // every buffer below is addressed at voice v of this batch
+  if (!in_bounds(hdr, v, batch)) return;
+  const VoiceFF& V = s.V;
+  load_tables(s.T, vc.T);
+  __syncthreads();
+  if (tid < kNumParams) {
+    const float u = fminf(fmaxf(params[(size_t)v * kNumParams + tid], 0.f), 1.f);
+    s.y[tid] = range_map_ff(u, vc.map_base[tid], vc.map_scale[tid], vc.map_curve[tid],
+                            vc.map_code[tid], vc.sym[tid], s.T);
+    b.y[(size_t)v * 80 + tid] = ff_to_float(s.y[tid]);
+  }
+  __syncthreads();
+  if (tid < 16) {
+    voice_ff_fill(s.V, s.y, tid);
+  } else if (tid == 32) {
+    const float l0 = ff_to_float(s.y[kMix]), l1 = ff_to_float(s.y[kMix + 1]),
+                l2 = ff_to_float(s.y[kMix + 2]);
+    const float inv = 1.f / fmaxf(1.f, l0 + l1 + l2);
+    *reinterpret_cast<float4*>(b.mix + (size_t)v * 4) =
+        make_float4(l0 * inv, l1 * inv, l2 * inv, ff_to_float(s.y[kSqr + 3]));
+  } else if (tid >= 64 && tid < 68) {
+    const int slot[4] = {kLfo + 2, kLfo + 8 + 2, kSine + 2, kSqr + 2};
+    s.p0[tid - 64] = ff_to_fix64(ff_mul(s.y[slot[tid - 64]], vc.inv_2pi));
+  }
+  __syncthreads();
+  if (tid < 6) s.V.level_d[tid] = gate_level_ff(tid, V, s.T);
+  __syncthreads();
+  unsigned long long lfo_carry = s.p0[half], vco_carry = s.p0[2 + half];
+  for (int base = 0; base < K; base += kCP - 1) {
+    const int nseg = min(kCP - 1, K - base);  // points base .. base + nseg
+    for (int i = tid; i < 6 * kCP; i += kCT) {
+      const int a = i / kCP, k = i % kCP;
+      if (k > nseg || !in_bounds(hdr, base + k, P)) continue;
+      const ff e = adsr_ff(ff_mul_f(vc.inv_cr, (float)(base + k)), a, V, s.T);
+      s.env[a][k] = e;
+      b.env[((size_t)v * 6 + a) * P + base + k] = ff_to_float(e);
+    }
+    __syncthreads();
+    unsigned long long inc = 0, tot;
+    if (p < nseg) {
+      const ff rate = ff_min(ff_max(ff_add(V.lfo_freq[half], ff_mul(V.lfo_depth[half], s.env[2 + 2 * half][p])),
+                                    ff_make(0.f)),
+                             ff_make((float)kLfoMaxHz));
+      inc = ff_to_fix64(ff_mul(rate, vc.inv_cr));
+    }
+    const unsigned long long theta = lfo_carry + half_scan(s, inc, tot);
+    lfo_carry += tot;
+    if (p <= nseg) {
+      const ff th = fix64_to_ff(theta);
+      b.phase[((size_t)v * 2 + half) * P + base + p] = ff_to_float(th);
+      s.env[3 + 2 * half][p] = lfo_ff(th, half, s.env[3 + 2 * half][p], V, s.T);
+    }
+    __syncthreads();
+    if (p <= nseg) {
+      const ff src[4] = {s.env[0][p], s.env[1][p], s.env[3][p], s.env[5][p]};
+      ff m = V.pitch_base[half];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) m = ff_add(m, ff_mul(V.pitch_w[half][q], src[q]));
+      s.env[2 + 2 * half][p] = m;
+      // the mixer's outputs as floats, two or three a half: the pitch one, then amplitudes
+      auto put = [&](int j, const float w[4]) {
+        float acc = w[0] * ff_to_float(src[0]);
+#pragma unroll
+        for (int q = 1; q < 4; ++q) acc = fmaf(w[q], ff_to_float(src[q]), acc);
+        b.dest[((size_t)v * 5 + j) * P + base + p] = acc;
+      };
+      const int jp = 2 * half;
+      float wp[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) wp[q] = ff_to_float(V.mod_w[q][jp]) * ff_to_float(V.inv_norm[jp]);
+      put(jp, wp);
+      put(jp + 1, V.amp_w[half]);
+      if (half == 1) put(4, V.amp_w[2]);
+    }
+    __syncthreads();
+    ff adv = ff_make(0.f);
+    SegVco sv;
+    if (p < nseg) {
+      const int k = base + p;
+      const int64_t rem = vc.n_samples - (int64_t)k * vc.R;
+      const int Rk = rem < vc.R ? (int)rem : vc.R;
+      float inc_first;
+      adv = vco_interval_ff(s.env[2 + 2 * half][p], s.env[2 + 2 * half][p + 1], (float)vc.R, Rk,
+                            vc.inv_R, vc.ln2_12R, vc.m_nyq_ff, vc.log2_440_over_sr, s.T, &sv,
+                            &inc_first);
+      if (half == 1) {  // drive 1 + SR / (8 f) at the (capped) frequency of the interval start
+        const float kap = fminf((float)kBrightnessMax, 1.f + 0.125f / inc_first);
+        b.kappa[((size_t)v * 2 + 0) * K + k] = kap;
+        b.kappa[((size_t)v * 2 + 1) * K + k] = 1.f / tanhf(kap);
+      }
+    }
+    const unsigned long long start =
+        vco_carry + half_scan(s, p < nseg ? ff_to_fix64(adv) : 0ull, tot);
+    vco_carry += tot;
+    if (p < nseg && in_bounds(hdr, base + p, K)) {
+      sv.phase0 = fix64_to_float(start);
+      b.seg[((size_t)v * 2 + half) * K + base + p] = sv;
+    }
+    __syncthreads();  // the chunk's envelopes are done with
+  }
+}
+
+// ---------------------------------------------------------------------------
+// 2. audio-rate reverse pass. Eight lanes take a control interval (R <= 128), lane
+// l its samples 16 l .. 16 l + 15, from the last to the first, so that the sum of
+// d/d(phase) over later samples is at hand: over the lane's own it runs along,
+// over the later lanes' it enters the moments afterwards (they are linear in it).
+// ---------------------------------------------------------------------------
+constexpr int kST = 128;
+constexpr int kSI = kST / 8;  // intervals per block
+
+// Phases (cycles) and increments of samples j0 .. j0 + 3; the increment of a
+// sample whose pitch is capped at Nyquist as 0 (it does not move with the pitch).
+__device__ __forceinline__ void vco_quad_and_inc(const SegVco& s, int j0, float ph[4], float inc[4]) {
+  vco_quad(s, j0, ph);
+  const int jc = s.jc_flags & 0xffff;
+  if (j0 + 3 < jc || j0 >= jc) {  // inside one piece: the increments are geometric
+    const bool in_b = j0 >= jc;
+    const float c = in_b ? s.cB : s.cA;
+    const bool lin = (s.jc_flags >> (in_b ? 17 : 16)) & 1;
+    const bool cap = (s.jc_flags >> (in_b ? 19 : 18)) & 1;
+    const float z = (float)(j0 - (in_b ? jc : 0)) * (lin ? 0.f : s.x);
+    const float r = lin ? 1.f : s.q2 - 1.f;
+    inc[0] = cap ? 0.f : fmaf(c, expm1_phase(z), c);
+    inc[1] = inc[0] * r;
+    inc[2] = inc[1] * r;
+    inc[3] = inc[2] * r;
+  } else {
+    bool cap[4];
+    vco_inc_quad(s, j0, inc, cap);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) inc[i] = cap[i] ? 0.f : inc[i];
+  }
+}
+
+__global__ void __launch_bounds__(kST) bwd_samples(const __grid_constant__ VoiceConst vc,
                                                    uint64_t seed, uint64_t batch_index, int batch,
-                                                   const float* __restrict__ mixc,
-                                                   const ff* __restrict__ dest,
-                                                   const SegVco* __restrict__ seg,
-                                                   const float* __restrict__ kappa,
                                                    const float* __restrict__ grad_audio,
-                                                   float* __restrict__ stat, ScratchHeader* hdr) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+                                                   const AdjBuffers b, ScratchHeader* hdr) {
+  const int lane = threadIdx.x & 31, l8 = lane & 7;
   const int v = blockIdx.y;
   const int K = vc.K, P = K + 1, R = vc.R;
-  const int k = blockIdx.x * (kBT / 32) + warp;
-  if (k >= K) return;
+  const int ki = blockIdx.x * kSI + (threadIdx.x >> 3);
+  if (ki - (lane >> 3) >= K) return;  // the warp's first interval is past the end
+  const bool valid = ki < K;
+  const int k = valid ? ki : K - 1;
   // the interval's control points k and k + 1, its descriptions and its row
   // of statistics belong to voice v of this batch
   if (!in_bounds(hdr, v, batch) || !in_bounds(hdr, k + 1, P)) return;
   const int64_t N = vc.n_samples;
-  // mixer gains and square-saw shape as the control pass stored them (the
-  // FP64 quotients rounded to float: no FP64 arithmetic in this kernel)
-  const float* mc = mixc + (size_t)v * 5;
-  const float g[3] = {mc[0], mc[1], mc[2]};
-  const float sigma = mc[3];
-  const float ip = 1.f / (1.f + sigma);
-  const int dj[3] = {1, 3, 4};
-  float a0[3], a1[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    a0[c] = ff_to_float(dest[((size_t)v * 5 + dj[c]) * P + k]);
-    a1[c] = ff_to_float(dest[((size_t)v * 5 + dj[c]) * P + k + 1]);
-  }
-  const SegVco s0 = seg[((size_t)v * 2 + 0) * K + k];
-  const SegVco s1 = seg[((size_t)v * 2 + 1) * K + k];
-  const float kap = kappa[((size_t)v * 2 + 0) * K + k];
-  const float itk = kappa[((size_t)v * 2 + 1) * K + k];
-  const int64_t rem = N - (int64_t)k * R;
-  const int Rk = rem < R ? (int)rem : R;
+  const float4 mx = *reinterpret_cast<const float4*>(b.mix + (size_t)v * 4);
+  const float sigma = mx.w, ip = 1.f / (1.f + sigma);
+  const float* d1 = b.dest + ((size_t)v * 5 + 1) * P + k;
+  const float a0[3] = {d1[0], d1[2 * P], d1[3 * P]};  // destinations 1, 3, 4
+  const float da[3] = {d1[1] - a0[0], d1[2 * P + 1] - a0[1], d1[3 * P + 1] - a0[2]};
+  const SegVco& s0 = b.seg[((size_t)v * 2 + 0) * K + k];
+  const SegVco& s1 = b.seg[((size_t)v * 2 + 1) * K + k];
+  const float kap = b.kappa[((size_t)v * 2 + 0) * K + k];
+  const float itk = b.kappa[((size_t)v * 2 + 1) * K + k];
+  const int64_t n_first = (int64_t)k * R;
+  const int Rk = valid ? (int)min((int64_t)R, N - n_first) : 0;
   const float invR = 1.f / (float)R;
   const uint64_t gv = batch_index * (uint64_t)batch + (uint64_t)v;
+  const uint2 key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
+  const float* ga = grad_audio + (size_t)v * N + n_first;
+  const bool vec = (N & 3) == 0 && (reinterpret_cast<uintptr_t>(grad_audio) & 15) == 0;
 
-  float acc[kStat];
+  float acc[24];
 #pragma unroll
-  for (int i = 0; i < kStat; ++i) acc[i] = 0.f;
-  float dphi[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-  float inc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-  bool capd[2][4] = {{false, false, false, false}, {false, false, false, false}};
-  const int j0 = 4 * lane;
-  const bool active = j0 < Rk;
-  if (active) {
-    float ps[4], pq[4];
-    vco_quad(s0, j0, ps);
-    vco_quad(s1, j0, pq);
-    vco_inc_quad(s0, j0, inc[0], capd[0]);
-    vco_inc_quad(s1, j0, inc[1], capd[1]);
-    const int64_t n0 = (int64_t)k * R + j0;
-    const uint4 nz = philox4x32_10(
-        make_uint4((uint32_t)gv, (uint32_t)(gv >> 32), (uint32_t)(n0 >> 2), kStreamNoise),
-        make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)));
+  for (int i = 0; i < 24; ++i) acc[i] = 0.f;
+  float ls[2] = {0.f, 0.f};  // sum of d/d(phase) over the lane's later samples
+#pragma unroll 1
+  for (int i = 3; i >= 0; --i) {
+    const int j0 = 4 * (4 * l8 + i);
+    if (j0 >= Rk) continue;
+    float ps[4], pq[4], inc[2][4], go4[4];
+    vco_quad_and_inc(s0, j0, ps, inc[0]);
+    vco_quad_and_inc(s1, j0, pq, inc[1]);
+    const uint4 nz = philox4x32_10(make_uint4((uint32_t)gv, (uint32_t)(gv >> 32),
+                                              (uint32_t)((n_first + j0) >> 2), kStreamNoise),
+                                   key);
     const uint32_t nw[4] = {nz.x, nz.y, nz.z, nz.w};
+    if (vec && j0 + 3 < Rk && in_bounds(hdr, (long long)v * N + n_first + j0 + 3, (long long)batch * N)) {
+      const float4 t = __ldg(reinterpret_cast<const float4*>(ga + j0));
+      go4[0] = t.x; go4[1] = t.y; go4[2] = t.z; go4[3] = t.w;
+    } else {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int j = j0 + i;
-      if (j >= Rk) {
-        inc[0][i] = inc[1][i] = 0.f;
-        continue;
-      }
-      const float go = in_bounds(hdr, (long long)v * N + n0 + i, (long long)batch * N)
-                           ? grad_audio[(size_t)v * N + n0 + i]
-                           : 0.f;
-      const float fj = (float)j * invR;
+      for (int t = 0; t < 4; ++t)
+        go4[t] = j0 + t < Rk && in_bounds(hdr, (long long)v * N + n_first + j0 + t, (long long)batch * N)
+                     ? ga[j0 + t]
+                     : 0.f;
+    }
+#pragma unroll
+    for (int t = 3; t >= 0; --t) {
+      const bool on = j0 + t < Rk;
+      const float go = go4[t];
+      const float fj = (float)(j0 + t) * invR;
       float A[3];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) A[c] = fmaf(fj, a1[c] - a0[c], a0[c]);
+      for (int c = 0; c < 3; ++c) A[c] = fmaf(fj, da[c], a0[c]);
       // SFU sine, cosine and tanh, as in the forward render
-      float xs, xc;
-      __sincosf(kTwoPiF * ps[i], &xs, &xc);
-      float sn, cs;
-      __sincosf(kTwoPiF * pq[i], &sn, &cs);
+      float xs, xc, sn, cs;
+      __sincosf(kTwoPiF * ps[t], &xs, &xc);
+      __sincosf(kTwoPiF * pq[t], &sn, &cs);
       const float th = tanh_from_y(kTwoLog2e * kap * sn);
       const float shp = fmaf(sigma, cs, 1.f);
-      const float xq = th * itk * shp * ip;
-      const float xn = fmaf(2.f, u01f(nw[i]), -1.f);
-      const float x[3] = {xs, xq, xn};
+      const float x[3] = {xs, th * itk * shp * ip, fmaf(2.f, u01f(nw[t]), -1.f)};
+      const float gg[3] = {go * mx.x, go * mx.y, go * mx.z};
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        const float dA = go * g[c] * x[c];
-        acc[10 + c] += dA * (1.f - fj);
-        acc[13 + c] += dA * fj;
-        acc[17 + c] += go * A[c] * x[c];
+        const float dA = gg[c] * x[c];
+        acc[10 + c] = fmaf(dA, 1.f - fj, acc[10 + c]);
+        acc[13 + c] = fmaf(dA, fj, acc[13 + c]);
+        acc[17 + c] = fmaf(go * A[c], x[c], acc[17 + c]);
       }
-      dphi[0][i] = go * g[0] * A[0] * kTwoPiF * xc;
       const float sech2 = 1.f - th * th;
-      const float dxq_dth = itk * ip * (kap * cs * sech2 * shp - th * sigma * sn);
-      dphi[1][i] = go * g[1] * A[1] * kTwoPiF * dxq_dth;
+      const float gA1 = gg[1] * A[1] * ip;
+      const float dphi[2] = {gg[0] * A[0] * kTwoPiF * xc,
+                             gA1 * kTwoPiF * itk * (kap * cs * sech2 * shp - th * sigma * sn)};
       // d xq / d kappa with d(1/tanh k)/dk = 1 - (1/tanh k)^2
-      acc[16] += go * g[1] * A[1] * ip * shp * (sn * sech2 * itk + th * (1.f - itk * itk));
-      acc[20] += go * g[1] * A[1] * th * itk * (cs - 1.f) * ip * ip;
+      acc[16] = fmaf(gA1 * shp, sn * sech2 * itk + th * (1.f - itk * itk), acc[16]);
+      acc[20] = fmaf(gA1 * ip * th * itk, cs - 1.f, acc[20]);
+#pragma unroll
+      for (int o = 0; o < 2; ++o) {
+        const float w = on ? inc[o][t] : 0.f, wr = w * fj, wl = w - wr;
+        acc[5 * o + 1] = fmaf(wl, ls[o], acc[5 * o + 1]);
+        acc[5 * o + 2] += wl;
+        acc[5 * o + 3] = fmaf(wr, ls[o], acc[5 * o + 3]);
+        acc[5 * o + 4] += wr;
+        ls[o] += dphi[o];
+      }
     }
   }
-  // reverse phase scan inside the interval: LS_j = sum of dphi over samples
-  // after j in this interval
+  // the later lanes' samples: their sum enters M1 and M2 times F1 and F2
 #pragma unroll
   for (int o = 0; o < 2; ++o) {
-    const float lt = dphi[o][0] + dphi[o][1] + dphi[o][2] + dphi[o][3];
-    float suf = lt;  // inclusive suffix over lanes >= lane
+    float suf = ls[o];  // inclusive over lanes >= l8 of the interval
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const float t = __shfl_down_sync(0xffffffffu, suf, d);
-      if (lane + d < 32) suf += t;
+    for (int d = 1; d < 8; d <<= 1) {
+      const float t = __shfl_down_sync(0xffffffffu, suf, d, 8);
+      if (l8 + d < 8) suf += t;
     }
-    float after = __shfl_down_sync(0xffffffffu, suf, 1);
-    if (lane == 31) after = 0.f;
-    float ls = after;  // strict suffix, walking from sample 3 down to 0
-    float M1 = 0.f, F1 = 0.f, M2 = 0.f, F2 = 0.f;
-#pragma unroll
-    for (int i = 3; i >= 0; --i) {
-      const int j = j0 + i;
-      if (active && j < Rk && !capd[o][i]) {
-        const float fj = (float)j * invR;
-        const float wl = inc[o][i] * (1.f - fj), wr = inc[o][i] * fj;
-        M1 += wl * ls;
-        F1 += wl;
-        M2 += wr * ls;
-        F2 += wr;
-      }
-      ls += dphi[o][i];
-    }
-    acc[5 * o + 0] += lt;
-    acc[5 * o + 1] += M1;
-    acc[5 * o + 2] += F1;
-    acc[5 * o + 3] += M2;
-    acc[5 * o + 4] += F2;
+    float after = __shfl_down_sync(0xffffffffu, suf, 1, 8);
+    if (l8 == 7) after = 0.f;
+    acc[5 * o + 0] = ls[o];
+    acc[5 * o + 1] = fmaf(after, acc[5 * o + 2], acc[5 * o + 1]);
+    acc[5 * o + 3] = fmaf(after, acc[5 * o + 4], acc[5 * o + 3]);
   }
-  // butterfly reduce-scatter of the kStat (<= 32) sums over the warp: at
-  // step s a lane keeps half of its slots (the upper half when bit s of its
-  // lane index is set) and adds its partner's copy of that half; after 31
-  // shuffles lane i holds the warp's total of sum i (instead of 5 shuffles
-  // for each of the kStat sums)
-  static_assert(kStat <= 32, "one sum per lane");
-  float r[32];
+  // butterfly reduce-scatter of the 21 (of 24) sums over the 8 lanes: at each step a
+  // lane keeps half of its slots and adds its partner's copy of that half; in
+  // the end lane l holds the totals of sums 3 l .. 3 l + 2
+  static_assert(kStat <= 24, "three sums per lane");
 #pragma unroll
-  for (int i = 0; i < 32; ++i) r[i] = i < kStat ? acc[i] : 0.f;
-#pragma unroll
-  for (int sh = 16; sh >= 1; sh >>= 1) {
+  for (int sh = 4, n = 12; sh >= 1; sh >>= 1, n >>= 1) {
     const bool up = (lane & sh) != 0;
 #pragma unroll
-    for (int i = 0; i < sh; ++i) {
-      const float send = up ? r[i] : r[i + sh];
-      const float keep = up ? r[i + sh] : r[i];
-      r[i] = keep + __shfl_xor_sync(0xffffffffu, send, sh);
+    for (int i = 0; i < n; ++i) {
+      const float send = up ? acc[i] : acc[i + n];
+      const float keep = up ? acc[i + n] : acc[i];
+      acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, sh);
     }
   }
-  if (lane < kStat) stat[((size_t)v * K + k) * kStat + lane] = r[0];
-}
-
-// ---------------------------------------------------------------------------
-// 3. reverse scan over intervals and the per-point pitch / amplitude adjoints.
-// One block per voice. gpt[half][v][k] = {dm_sine, dm_sq, dA_sine, dA_sq,
-// dA_noise}: half 0 from interval k (point k its left end), half 1 from
-// interval k - 1 (its right end); the point's adjoint is their sum.
-// vacc[v] = {dphase0_sine, dphase0_sq (cycles), dg0, dg1, dg2, dshape, 0, 0}.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kBT) bwd_interval_scan(const __grid_constant__ VoiceConst vc,
-                                                         const float* __restrict__ stat,
-                                                         const SegVco* __restrict__ seg,
-                                                         const float* __restrict__ kappa,
-                                                         double* __restrict__ gpt,
-                                                         double* __restrict__ vacc,
-                                                         ScratchHeader* hdr) {
-  __shared__ double warp_tot[2 * (kBT / 32)];
-  __shared__ double red[8][kBT / 32];
-  const int v = blockIdx.x;
-  const int K = vc.K, P = K + 1;
-  const double l12 = kLn2 / 12.0;
-  double carry0 = 0.0, carry1 = 0.0;
-  double part[4] = {0.0, 0.0, 0.0, 0.0};  // dg0, dg1, dg2, dshape
-  double* gv = gpt + (size_t)v * P * 5;
-  for (int base = 0; base < K; base += kBT) {
-    const int idx = K - 1 - (base + (int)threadIdx.x);  // reversed order
-    const bool ok = idx >= 0;
-    const float* st = stat + ((size_t)v * K + (ok ? idx : 0)) * kStat;
-    double t0 = ok ? (double)st[0] : 0.0, t1 = ok ? (double)st[5] : 0.0;
-    double e0 = t0, e1 = t1, tot0, tot1;
-    block_exclusive_scan2<double, kBT>(e0, e1, warp_tot, tot0, tot1);
-    if (ok) {
-      // C_{idx+1}: sum of d/d(phase) over all later intervals
-      const double c0 = carry0 + e0, c1 = carry1 + e1;
-      const double dl0 = l12 * ((double)st[1] + (double)st[2] * c0);
-      const double dr0 = l12 * ((double)st[3] + (double)st[4] * c0);
-      const double dl1 = l12 * ((double)st[6] + (double)st[7] * c1);
-      const double dr1 = l12 * ((double)st[8] + (double)st[9] * c1);
-      // square-saw drive kappa_k = min(50, 1 + SR/(8 f_k)): d kappa / d m =
-      // -(kappa - 1) ln2/12 while below the bound and the pitch is uncapped
-      const SegVco s1 = seg[((size_t)v * 2 + 1) * K + idx];
-      const float kap = kappa[((size_t)v * 2 + 0) * K + idx];
-      double dk = 0.0;
-      if (kap < (float)kBrightnessMax && !((s1.jc_flags >> 18) & 1))
-        dk = (double)st[16] * (-(double)(kap - 1.f) * l12);
-      // interval idx reaches points idx (left end) and idx + 1 (right end):
-      // the left parts go to gv, the right parts to gr, one store each; the
-      // consumer adds the two halves of a point
-      double* gl = gv + (size_t)idx * 5;
-      double* gr = gv + (size_t)P * 5 * gridDim.x + (size_t)(idx + 1) * 5;
-      if (in_bounds(hdr, idx + 1, P)) {  // both halves stay in the voice's P points
-        gl[0] = dl0;
-        gr[0] = dr0;
-        gl[1] = dl1 + dk;
-        gr[1] = dr1;
-        for (int c = 0; c < 3; ++c) {
-          gl[2 + c] = (double)st[10 + c];
-          gr[2 + c] = (double)st[13 + c];
-        }
-      }
-      for (int c = 0; c < 4; ++c) part[c] += (double)st[17 + c];
-    }
-    carry0 += tot0;
-    carry1 += tot1;
-  }
-  // per-voice sums of the gain / shape partials
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int c = 0; c < 4; ++c) {
-    const double w = warp_sum_d(part[c]);
-    if (lane == 0) red[c][warp] = w;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double* va = vacc + (size_t)v * 8;
-    va[0] = carry0;  // sum over every sample: d/d(initial phase, cycles)
-    va[1] = carry1;
-    for (int c = 0; c < 4; ++c) {
-      double s = 0.0;
-      for (int w = 0; w < kBT / 32; ++w) s += red[c][w];
-      va[2 + c] = s;
-    }
-    va[6] = va[7] = 0.0;
+  if (valid && l8 < kStat / 3) {
+    float* st = b.stat + ((size_t)v * K + k) * kStat + 3 * l8;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) st[i] = acc[i];
   }
 }
 
 // ---------------------------------------------------------------------------
-// 4. control-rate reverse sweep, one block per voice, in FP32: a gradient
-// needs a relative accuracy of about 1e-3, not the forward's float-float (the
-// forward values it differentiates at are recomputed in float-float and FP64
-// and rounded to float here).
+// 3. reverse scan over intervals (FP64) and control-rate reverse sweep, one block
+// per voice; the sweep in FP32: a gradient needs a relative accuracy of about
+// 1e-3, not the forward's float-float (the forward values it differentiates at
+// are recomputed in float-float and rounded to float).
 // ---------------------------------------------------------------------------
 constexpr int kGY = 80;  // slots of the per-voice human-range gradient d/dy (78 used)
 constexpr int kBC = 512;  // threads of the control-rate reverse sweep (one block per voice)
@@ -399,6 +502,25 @@ __device__ __forceinline__ void acc_y(float* gy_warp, int slot, float val) {
   if ((threadIdx.x & 31) == 0) gy_warp[slot] += w;
 }
 
+// Adds 32 values of each lane up over the warp and lane i's total of value i to
+// the warp's row at slot(i): a butterfly reduce-scatter of 31 shuffles.
+template <class Slot>
+__device__ __forceinline__ void acc_y32(float* gy_warp, float (&r)[32], Slot slot) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int sh = 16; sh >= 1; sh >>= 1) {
+    const bool up = (lane & sh) != 0;
+#pragma unroll
+    for (int i = 0; i < sh; ++i) {
+      const float send = up ? r[i] : r[i + sh];
+      const float keep = up ? r[i + sh] : r[i];
+      r[i] = keep + __shfl_xor_sync(0xffffffffu, send, sh);
+    }
+  }
+  gy_warp[slot(lane)] += r[0];
+  __syncwarp();
+}
+
 // d y / d u of the range map for parameter p at u (FP32: the FP64 pipe is
 // narrow on this GPU, and the gradient needs ~1e-6).
 __device__ __forceinline__ float range_map_dydu(const VoiceConst& vc, int p, float u_raw) {
@@ -411,14 +533,7 @@ __device__ __forceinline__ float range_map_dydu(const VoiceConst& vc, int p, flo
 }
 
 __global__ void __launch_bounds__(kBC) bwd_control(const __grid_constant__ VoiceConst vc,
-                                                   const double* __restrict__ y,
-                                                   const ff* __restrict__ env,
-                                                   const double* __restrict__ lfo_phase,
-                                                   const ff* __restrict__ dest,
-                                                   const double* __restrict__ gpt,
-                                                   const double* __restrict__ vacc,
-                                                   float* __restrict__ dtheta,
-                                                   float* __restrict__ denv,
+                                                   const AdjBuffers buf,
                                                    const float* __restrict__ u_in,
                                                    float* __restrict__ grad_params,
                                                    int batch, ScratchHeader* hdr) {
@@ -426,13 +541,42 @@ __global__ void __launch_bounds__(kBC) bwd_control(const __grid_constant__ Voice
   __shared__ float gyw_all[kBC / 32][kGY];  // per-warp partial gradients
   __shared__ float yv[kNumParams];
   __shared__ float warp_tot[2 * (kBC / 32)];
+  __shared__ double warp_totd[2 * (kBC / 32)];
+  __shared__ double red[4][kBC / 32];
   const int v = blockIdx.x;
-  const int P = vc.K + 1;
+  const int K = vc.K, P = K + 1;
+  if (!in_bounds(hdr, v, batch)) return;
   const float inv_cr = (float)(1.0 / vc.control_rate);
   const float inv_2pi = 0.15915494309189533577f;
+  const float l12 = (float)(kLn2 / 12.0);
   float* gyw = gyw_all[threadIdx.x >> 5];
   for (int i = threadIdx.x; i < kGY * (kBC / 32); i += kBC) (&gyw_all[0][0])[i] = 0.f;
-  for (int i = threadIdx.x; i < kNumParams; i += kBC) yv[i] = (float)y[(size_t)v * kNumParams + i];
+  for (int i = threadIdx.x; i < kNumParams; i += kBC) yv[i] = buf.y[(size_t)v * 80 + i];
+  const float* stat = buf.stat + (size_t)v * K * kStat;
+  double2* csum = buf.csum + (size_t)v * K;
+  // C_{idx+1}: sum of d/d(phase) over all later intervals; and the voice's sums
+  // of the gain and shape partials
+  double total0 = 0.0, total1 = 0.0;
+  {
+    double part[4] = {0.0, 0.0, 0.0, 0.0};  // dg0, dg1, dg2, dshape
+    for (int base = 0; base < K; base += kBC) {
+      const int idx = K - 1 - (base + (int)threadIdx.x);  // reversed order
+      const bool ok = idx >= 0;
+      const float* st = stat + (size_t)(ok ? idx : 0) * kStat;
+      double e0 = ok ? (double)st[0] : 0.0, e1 = ok ? (double)st[5] : 0.0, t0, t1;
+      if (ok)
+        for (int c = 0; c < 4; ++c) part[c] += (double)st[17 + c];
+      block_exclusive_scan2<double, kBC>(e0, e1, warp_totd, t0, t1);
+      if (ok && in_bounds(hdr, idx, K)) csum[idx] = make_double2(total0 + e0, total1 + e1);
+      total0 += t0;
+      total1 += t1;
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int c = 0; c < 4; ++c) {
+      const double w = warp_sum_d(part[c]);
+      if (lane == 0) red[c][warp] = w;
+    }
+  }
   __syncthreads();
   float inv_norm[5], wsum_col[5];
   for (int j = 0; j < 5; ++j) {
@@ -447,10 +591,9 @@ __global__ void __launch_bounds__(kBC) bwd_control(const __grid_constant__ Voice
     for (int s = 0; s < 5; ++s) ws += yv[kLfo + 8 * l + 3 + s];
     lfo_wsum[l] = ws;
   }
-  const double* gv = gpt + (size_t)v * P * 5;
-  const double* gvr = gv + (size_t)P * 5 * gridDim.x;  // the right-end halves
-  float* dth = dtheta + (size_t)v * 2 * P;
-  float* de = denv + (size_t)v * 6 * P;
+  float* dth = buf.dtheta + (size_t)v * 2 * P;
+  float* de = buf.denv + (size_t)v * 6 * P;
+  const float* env = buf.env + (size_t)v * 6 * P;
 
   // pass A: modulation mixer, LFO outputs, pitch
   for (int base = 0; base < P; base += kBC) {
@@ -458,61 +601,82 @@ __global__ void __launch_bounds__(kBC) bwd_control(const __grid_constant__ Voice
     const bool ok = k < P;
     const int kk = ok ? k : 0;
     float e[6];
-    for (int a = 0; a < 6; ++a) e[a] = ff_to_float(env[((size_t)v * 6 + a) * P + kk]);
+    for (int a = 0; a < 6; ++a) e[a] = env[(size_t)a * P + kk];
     float mix[2], sh[2][5], dsh[2][5], lfo[2];
     for (int l = 0; l < 2; ++l) {
-      const float th = (float)lfo_phase[((size_t)v * 2 + l) * P + kk];
-      lfo_shapes(th, sh[l], dsh[l]);
+      lfo_shapes(buf.phase[((size_t)v * 2 + l) * P + kk], sh[l], dsh[l]);
       float accm = 0.f;
       for (int s = 0; s < 5; ++s) accm += yv[kLfo + 8 * l + 3 + s] * sh[l][s];
       mix[l] = lfo_wsum[l] < 1e-12f ? 0.f : accm / lfo_wsum[l];
       lfo[l] = e[3 + 2 * l] * mix[l];
     }
     const float src[4] = {e[0], e[1], lfo[0], lfo[1]};
-    float dd[5] = {0, 0, 0, 0, 0}, dst[5];
+    // the point's pitch and amplitude adjoints: the left end of interval k and the
+    // right end of interval k - 1
     float gk[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-    if (ok)
-      for (int j = 0; j < 5; ++j) gk[j] = (float)(gv[(size_t)k * 5 + j] + gvr[(size_t)k * 5 + j]);
-    if (ok) {
-      dd[0] = yv[kSine + 1] * gk[0];
-      dd[2] = yv[kSqr + 1] * gk[1];
-      dd[1] = gk[2];
-      dd[3] = gk[3];
-      dd[4] = gk[4];
+    if (ok && k < K) {
+      const float* st = stat + (size_t)k * kStat;
+      const double2 c = csum[k];
+      gk[0] = l12 * (float)((double)st[1] + (double)st[2] * c.x);
+      gk[1] = l12 * (float)((double)st[6] + (double)st[7] * c.y);
+      // square-saw drive kappa_k = min(50, 1 + SR/(8 f_k)): d kappa / d m =
+      // -(kappa - 1) ln2/12 while below the bound and the pitch is uncapped
+      const float kap = buf.kappa[((size_t)v * 2 + 0) * K + k];
+      if (kap < (float)kBrightnessMax &&
+          !((buf.seg[((size_t)v * 2 + 1) * K + k].jc_flags >> 18) & 1))
+        gk[1] += st[16] * (-(kap - 1.f) * l12);
+      for (int c3 = 0; c3 < 3; ++c3) gk[2 + c3] = st[10 + c3];
     }
-    for (int j = 0; j < 5; ++j) dst[j] = ff_to_float(dest[((size_t)v * 5 + j) * P + kk]);
+    if (ok && k > 0) {
+      const float* st = stat + (size_t)(k - 1) * kStat;
+      const double2 c = csum[k - 1];
+      gk[0] += l12 * (float)((double)st[3] + (double)st[4] * c.x);
+      gk[1] += l12 * (float)((double)st[8] + (double)st[9] * c.y);
+      for (int c3 = 0; c3 < 3; ++c3) gk[2 + c3] += st[13 + c3];
+    }
+    const float dd[5] = {yv[kSine + 1] * gk[0], gk[2], yv[kSqr + 1] * gk[1], gk[3], gk[4]};
+    float dst[5];
+    for (int j = 0; j < 5; ++j) dst[j] = buf.dest[((size_t)v * 5 + j) * P + kk];
     // pitch: m = midi + tune + depth * dest
     const float dm0 = gk[0];
     const float dm1 = gk[1];
-    acc_y(gyw, kMidi, dm0 + dm1);
-    acc_y(gyw, kSine, dm0);
     acc_y(gyw, kSqr, dm1);
     acc_y(gyw, kSine + 1, dm0 * dst[0]);
     acc_y(gyw, kSqr + 1, dm1 * dst[2]);
+    // the other 32 sums in one go: 20 modulation weights, 10 shape weights, midi, sine tune
+    float r[32];
+    r[30] = dm0 + dm1;
+    r[31] = dm0;
     // dest_j = (sum_i W_ij src_i) / max(1, sum_i W_ij)
     float dsrc[4] = {0, 0, 0, 0};
+#pragma unroll
     for (int j = 0; j < 5; ++j) {
       const float over = wsum_col[j] > 1.f ? 1.f : 0.f;
+#pragma unroll
       for (int i = 0; i < 4; ++i) {
         dsrc[i] += dd[j] * yv[kMod + 5 * i + j] * inv_norm[j];
-        acc_y(gyw, kMod + 5 * i + j, dd[j] * (src[i] * inv_norm[j] - over * dst[j] * inv_norm[j]));
+        r[5 * i + j] = dd[j] * (src[i] * inv_norm[j] - over * dst[j] * inv_norm[j]);
       }
     }
     float dea[6] = {dsrc[0], dsrc[1], 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
     for (int l = 0; l < 2; ++l) {
       const float dl = dsrc[2 + l];
       dea[3 + 2 * l] = dl * mix[l];
       const float dmix = dl * e[3 + 2 * l];
       float dthv = 0.f;
-      if (lfo_wsum[l] >= 1e-12f) {
-        for (int s = 0; s < 5; ++s) {
-          acc_y(gyw, kLfo + 8 * l + 3 + s, dmix * (sh[l][s] - mix[l]) / lfo_wsum[l]);
-          dthv += yv[kLfo + 8 * l + 3 + s] * dsh[l][s];
-        }
-        dthv *= dmix / lfo_wsum[l];
+      const bool on = lfo_wsum[l] >= 1e-12f;
+#pragma unroll
+      for (int s = 0; s < 5; ++s) {
+        r[20 + 5 * l + s] = on ? dmix * (sh[l][s] - mix[l]) / lfo_wsum[l] : 0.f;
+        dthv += yv[kLfo + 8 * l + 3 + s] * dsh[l][s];
       }
-      if (ok) dth[(size_t)l * P + k] = dthv;
+      if (ok) dth[(size_t)l * P + k] = on ? dthv * (dmix / lfo_wsum[l]) : 0.f;
     }
+    acc_y32(gyw, r, [](int i) {
+      return i < 20 ? kMod + i : i < 25 ? kLfo + 3 + i - 20 : i < 30 ? kLfo + 8 + 3 + i - 25
+             : i == 30 ? kMidi : kSine;
+    });
     if (ok)
       for (int a = 0; a < 6; ++a) de[(size_t)a * P + k] = dea[a];
   }
@@ -530,7 +694,7 @@ __global__ void __launch_bounds__(kBC) bwd_control(const __grid_constant__ Voice
       float dinc = 0.f, er = 0.f, rate_raw = 0.f;
       if (ok) {
         dinc = (l == 0 ? carry0 + a0 : carry1 + a1);  // sum of dtheta over points after idx
-        er = ff_to_float(env[((size_t)v * 6 + 2 + 2 * l) * P + idx]);
+        er = env[(size_t)(2 + 2 * l) * P + idx];
         rate_raw = yv[kLfo + 8 * l] + yv[kLfo + 8 * l + 1] * er;
       }
       const bool inside = ok && rate_raw >= 0.f && rate_raw <= (float)kLfoMaxHz;
@@ -574,11 +738,12 @@ __global__ void __launch_bounds__(kBC) bwd_control(const __grid_constant__ Voice
       dur_acc += g * out[5];
     }
   }
+  float r[32];
 #pragma unroll
-  for (int a = 0; a < 6; ++a)
-#pragma unroll
-    for (int q = 0; q < 5; ++q) acc_y(gyw, kAdsr + 5 * a + q, acc[a][q]);
-  acc_y(gyw, kDuration, dur_acc);
+  for (int i = 0; i < 30; ++i) r[i] = acc[i / 5][i % 5];
+  r[30] = dur_acc;
+  r[31] = 0.f;
+  acc_y32(gyw, r, [](int i) { return i < 30 ? kAdsr + i : i == 30 ? kDuration : kGY - 1; });
   __syncthreads();
   for (int i = threadIdx.x; i < kGY; i += kBC) {
     float t = 0.f;
@@ -588,16 +753,21 @@ __global__ void __launch_bounds__(kBC) bwd_control(const __grid_constant__ Voice
   __syncthreads();
 
   if (threadIdx.x == 0) {
-    const double* va = vacc + (size_t)v * 8;
-    gy[kSine + 2] += (float)va[0] * inv_2pi;
-    gy[kSqr + 2] += (float)va[1] * inv_2pi;
-    gy[kSqr + 3] += (float)va[5];
+    gy[kSine + 2] += (float)total0 * inv_2pi;  // sums over every sample: d/d(initial phase, cycles)
+    gy[kSqr + 2] += (float)total1 * inv_2pi;
+    float va[4];
+    for (int c = 0; c < 4; ++c) {
+      double t = 0.0;
+      for (int w = 0; w < kBC / 32; ++w) t += red[c][w];
+      va[c] = (float)t;
+    }
+    gy[kSqr + 3] += va[3];
     // mixer gains g_i = l_i / max(1, sum l)
     const float l0 = yv[kMix], l1 = yv[kMix + 1], l2 = yv[kMix + 2];
     const float sum = l0 + l1 + l2, norm = fmaxf(1.f, sum);
-    const float dotg = (float)va[2] * l0 + (float)va[3] * l1 + (float)va[4] * l2;
+    const float dotg = va[0] * l0 + va[1] * l1 + va[2] * l2;
     for (int c = 0; c < 3; ++c)
-      gy[kMix + c] += (float)va[2 + c] / norm - (sum > 1.f ? dotg / (norm * norm) : 0.f);
+      gy[kMix + c] += va[c] / norm - (sum > 1.f ? dotg / (norm * norm) : 0.f);
   }
   __syncthreads();
   // through the range map: d/du = d/dy dy/du
@@ -612,7 +782,7 @@ __global__ void __launch_bounds__(kBC) bwd_control(const __grid_constant__ Voice
 }  // namespace
 
 size_t backward_workspace_bytes(const VoiceConst& vc, int batch) {
-  return bwd_layout(vc, batch, control_bytes(vc, batch)).total;
+  return adj_carve(vc, batch, nullptr).total;
 }
 
 cudaError_t launch_render_backward(const VoiceConst& vc, uint64_t seed, uint64_t batch_index,
@@ -620,23 +790,11 @@ cudaError_t launch_render_backward(const VoiceConst& vc, uint64_t seed, uint64_t
                                    float* grad_params, void* workspace, ScratchHeader* hdr,
                                    cudaStream_t st) {
   if (vc.R > 128) return cudaErrorInvalidValue;
-  const ControlBuffers cb = control_carve(vc, batch, workspace);
-  const BwdLayout L = bwd_layout(vc, batch, control_bytes(vc, batch));
-  char* ws = static_cast<char*>(workspace);
-  float* stat = reinterpret_cast<float*>(ws + L.stat);
-  double* gpt = reinterpret_cast<double*>(ws + L.gpt);
-  double* vacc = reinterpret_cast<double*>(ws + L.vacc);
-  float* dtheta = reinterpret_cast<float*>(ws + L.dtheta);
-  float* denv = reinterpret_cast<float*>(ws + L.denv);
-  const int K = vc.K, P = K + 1;
-  launch_control_fused(vc, seed, batch_index, batch, params, nullptr, cb, hdr, st);
-  cudaMemsetAsync(gpt, 0, sizeof(double) * 2 * (size_t)batch * P * 5, st);
-  dim3 gs((K + kBT / 32 - 1) / (kBT / 32), batch);
-  bwd_samples<<<gs, kBT, 0, st>>>(vc, seed, batch_index, batch, cb.mixc, cb.dest, cb.seg, cb.kappa,
-                                  grad_audio, stat, hdr);
-  bwd_interval_scan<<<batch, kBT, 0, st>>>(vc, stat, cb.seg, cb.kappa, gpt, vacc, hdr);
-  bwd_control<<<batch, kBC, 0, st>>>(vc, cb.y, cb.env, cb.lfo_phase, cb.dest, gpt, vacc, dtheta,
-                                     denv, params, grad_params, batch, hdr);
+  const AdjBuffers b = adj_carve(vc, batch, workspace);
+  bwd_recompute<<<batch, kCT, 0, st>>>(vc, batch, params, b, hdr);
+  const dim3 gs((vc.K + kSI - 1) / kSI, batch);
+  bwd_samples<<<gs, kST, 0, st>>>(vc, seed, batch_index, batch, grad_audio, b, hdr);
+  bwd_control<<<batch, kBC, 0, st>>>(vc, b, params, grad_params, batch, hdr);
   return cudaGetLastError();
 }
 

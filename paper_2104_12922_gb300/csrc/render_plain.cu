@@ -42,9 +42,7 @@ AudioLayout audio_layout(const VoiceConst& vc, int B, size_t base) {
   return L;
 }
 
-// The control modules' work per element, shared by the module kernels below
-// (one element per thread of a grid) and by control_fused_kernel (one CTA
-// per voice looping over the voice's elements), so both write the same bits.
+// The control modules' work per element.
 
 // Parameter module: draw (or read) and range-map parameter p of voice v.
 __device__ __forceinline__ void params_elem(const VoiceConst& vc, uint64_t seed,
@@ -106,84 +104,6 @@ __device__ __forceinline__ void lfo_rate_elem(const VoiceConst& vc, const VoiceF
     const ff rate = ff_min(ff_max(ff_add(V.lfo_freq[l], ff_mul(V.lfo_depth[l], e)), ff_make(0.f)),
                            ff_make((float)kLfoMaxHz));
     lfo_inc[((size_t)v * 2 + l) * P + k] = ff_to_double(ff_mul(rate, inv_cr));
-  }
-}
-
-// Synchronises the first kPT threads (warps 0 .. kPT/32 - 1) of a larger
-// block on named barrier 1: the phase scans of control_fused_kernel run on
-// those warps alone, with the module kernel's width and summation order.
-__device__ __forceinline__ void sync_scan_warps() {
-  asm volatile("bar.sync 1, %0;" ::"n"(kPT) : "memory");
-}
-
-// Exclusive block scan of two values over kPT threads (block_exclusive_scan2
-// of render_common.cuh, the same arithmetic and order), synchronised by
-// `sync`: __syncthreads in a block of kPT threads, sync_scan_warps in a
-// larger one.
-template <class Sync>
-__device__ __forceinline__ void scan2_kpt(double& a, double& b, double* warp_tot, double& tot_a,
-                                          double& tot_b, Sync sync) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double ia = a, ib = b;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    double na = __shfl_up_sync(0xffffffffu, ia, o);
-    double nb = __shfl_up_sync(0xffffffffu, ib, o);
-    if (lane >= o) { ia += na; ib += nb; }
-  }
-  if (lane == 31) { warp_tot[warp] = ia; warp_tot[kPT / 32 + warp] = ib; }
-  sync();
-  if (warp == 0) {
-    double wa = lane < kPT / 32 ? warp_tot[lane] : 0.0;
-    double wb = lane < kPT / 32 ? warp_tot[kPT / 32 + lane] : 0.0;
-#pragma unroll
-    for (int o = 1; o < kPT / 32; o <<= 1) {
-      double na = __shfl_up_sync(0xffffffffu, wa, o);
-      double nb = __shfl_up_sync(0xffffffffu, wb, o);
-      if (lane >= o) { wa += na; wb += nb; }
-    }
-    if (lane < kPT / 32) { warp_tot[lane] = wa; warp_tot[kPT / 32 + lane] = wb; }
-  }
-  sync();
-  const double pa = warp > 0 ? warp_tot[warp - 1] : 0.0;
-  const double pb = warp > 0 ? warp_tot[kPT / 32 + warp - 1] : 0.0;
-  tot_a = warp_tot[kPT / 32 - 1];
-  tot_b = warp_tot[2 * (kPT / 32) - 1];
-  double ea = __shfl_up_sync(0xffffffffu, ia, 1);
-  double eb = __shfl_up_sync(0xffffffffu, ib, 1);
-  if (lane == 0) { ea = 0.0; eb = 0.0; }
-  a = pa + ea;
-  b = pb + eb;
-  sync();
-}
-
-// Exclusive running sum of per-step phase increments, wrapped to [0,1),
-// starting from an initial phase: the two sequences of voice v, by kPT
-// threads (see scan2_kpt for `sync`).
-template <class Sync>
-__device__ __forceinline__ void phase_scan_block(const double* inc, double* phase, int len,
-                                                 int stride_seq, const double* y, int init_slot0,
-                                                 int init_slot1, int v, double* warp_tot,
-                                                 Sync sync) {
-  const double two_pi = 6.28318530717958647692;
-  const double* yv = y + (size_t)v * kNumParams;
-  double carry0 = wrap01(yv[init_slot0] / two_pi);
-  double carry1 = wrap01(yv[init_slot1] / two_pi);
-  const double* in0 = inc + (size_t)(2 * v) * stride_seq;
-  const double* in1 = inc + (size_t)(2 * v + 1) * stride_seq;
-  double* out0 = phase + (size_t)(2 * v) * stride_seq;
-  double* out1 = phase + (size_t)(2 * v + 1) * stride_seq;
-  for (int base = 0; base < len; base += kPT) {
-    const int i = base + threadIdx.x;
-    double a = i < len ? in0[i] : 0.0, b = i < len ? in1[i] : 0.0;
-    double ta, tb;
-    scan2_kpt(a, b, warp_tot, ta, tb, sync);
-    if (i < len) {
-      out0[i] = wrap01(carry0 + a);
-      out1[i] = wrap01(carry1 + b);
-    }
-    carry0 = wrap01(carry0 + ta);
-    carry1 = wrap01(carry1 + tb);
   }
 }
 
@@ -268,12 +188,32 @@ __global__ void plain_lfo_rate(const __grid_constant__ VoiceConst vc, const Voic
   lfo_rate_elem(vc, vff[v], env, lfo_inc, v, k);
 }
 
-// Running phase sums; one block scans the two sequences of a voice.
+// Exclusive running sums of per-step phase increments, wrapped to [0,1),
+// starting from an initial phase; one block scans the two sequences of a voice.
 __global__ void plain_phase_scan(const double* inc, double* phase, int len, int stride_seq,
                                  const double* y, int init_slot0, int init_slot1) {
   __shared__ double warp_tot[2 * (kPT / 32)];
-  phase_scan_block(inc, phase, len, stride_seq, y, init_slot0, init_slot1, blockIdx.x, warp_tot,
-                   [] { __syncthreads(); });
+  const double two_pi = 6.28318530717958647692;
+  const int v = blockIdx.x;
+  const double* yv = y + (size_t)v * kNumParams;
+  double carry0 = wrap01(yv[init_slot0] / two_pi);
+  double carry1 = wrap01(yv[init_slot1] / two_pi);
+  const double* in0 = inc + (size_t)(2 * v) * stride_seq;
+  const double* in1 = inc + (size_t)(2 * v + 1) * stride_seq;
+  double* out0 = phase + (size_t)(2 * v) * stride_seq;
+  double* out1 = phase + (size_t)(2 * v + 1) * stride_seq;
+  for (int base = 0; base < len; base += kPT) {
+    const int i = base + threadIdx.x;
+    double a = i < len ? in0[i] : 0.0, b = i < len ? in1[i] : 0.0;
+    double ta, tb;
+    block_exclusive_scan2<double, kPT>(a, b, warp_tot, ta, tb);
+    if (i < len) {
+      out0[i] = wrap01(carry0 + a);
+      out1[i] = wrap01(carry1 + b);
+    }
+    carry0 = wrap01(carry0 + ta);
+    carry1 = wrap01(carry1 + tb);
+  }
 }
 
 // LFO outputs and modulation mixer at the control points.
@@ -307,54 +247,6 @@ __global__ void plain_seg_phase(const __grid_constant__ VoiceConst vc, const dou
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (size_t)batch * 2 * vc.K) return;
   seg[i].phase0 = (float)seg_phase[i];
-}
-
-// The whole control pipeline of one voice per CTA (kFusedCtl threads): the
-// same steps and per-element code as the module kernels above, in the same
-// order, separated by barriers instead of launches; the two phase scans run
-// on the first kPT threads, as wide as the module kernel's and in its order,
-// so every buffer gets the same bits. The adjoint's forward recomputation
-// runs it: at its batch sizes the nine module launches are each a few
-// microseconds of mostly idle GPU.
-constexpr int kFusedCtl = 1024;
-__global__ void __launch_bounds__(kFusedCtl) control_fused_kernel(
-    const __grid_constant__ VoiceConst vc, uint64_t seed, uint64_t batch_index, int batch,
-    const float* params_in, float* params_out, const ControlBuffers cb, ScratchHeader* hdr) {
-  __shared__ FFTables T;
-  __shared__ ff yff[kNumParams];
-  __shared__ double warp_tot[2 * (kPT / 32)];
-  const int v = blockIdx.x, tid = threadIdx.x;
-  const int P = vc.K + 1, K = vc.K;
-  // every buffer below is addressed at voice v of this batch
-  if (!in_bounds(hdr, v, batch)) return;
-  load_tables(T, vc.T);
-  if (tid < kNumParams)
-    params_elem(vc, seed, batch_index, batch, params_in, params_out, cb.y, v, tid);
-  __syncthreads();
-  voice_consts_block(cb.y, cb.vff, cb.mixc, v, yff, T);
-  __syncthreads();
-  const VoiceFF& V = cb.vff[v];
-  for (int i = tid; i < 6 * P; i += kFusedCtl) adsr_elem(vc, V, T, cb.env, v, i);
-  __syncthreads();
-  for (int k = tid; k < P; k += kFusedCtl) lfo_rate_elem(vc, V, cb.env, cb.lfo_inc, v, k);
-  __syncthreads();
-  if (tid < kPT)
-    phase_scan_block(cb.lfo_inc, cb.lfo_phase, P, P, cb.y, kLfo + 2, kLfo + 8 + 2, v, warp_tot,
-                     sync_scan_warps);
-  __syncthreads();
-  for (int k = tid; k < P; k += kFusedCtl)
-    modmix_elem(vc, V, T, cb.env, cb.lfo_phase, cb.dest, v, k);
-  __syncthreads();
-  for (int k = tid; k < K; k += kFusedCtl)
-    if (in_bounds(hdr, k + 1, P))  // the interval's end point
-      vco_interval_elem(vc, V, T, cb.dest, cb.seg, cb.seg_sum, cb.kappa, v, k);
-  __syncthreads();
-  if (tid < kPT)
-    phase_scan_block(cb.seg_sum, cb.seg_start, K, K, cb.y, kSine + 2, kSqr + 2, v, warp_tot,
-                     sync_scan_warps);
-  __syncthreads();
-  for (int i = tid; i < 2 * K; i += kFusedCtl)
-    cb.seg[(size_t)v * 2 * K + i].phase0 = (float)cb.seg_start[(size_t)v * 2 * K + i];
 }
 
 // Upsampled amplitudes (VCA control inputs) at audio rate.
@@ -523,13 +415,6 @@ void launch_control_pipeline(const VoiceConst& vc, uint64_t seed, uint64_t batch
                                           kSqr + 2);
   plain_seg_phase<<<(int)(((size_t)batch * 2 * K + kPT - 1) / kPT), kPT, 0, st>>>(
       vc, cb.seg_start, cb.seg, batch);
-}
-
-void launch_control_fused(const VoiceConst& vc, uint64_t seed, uint64_t batch_index, int batch,
-                          const float* params_in, float* params_out, const ControlBuffers& cb,
-                          ScratchHeader* hdr, cudaStream_t st) {
-  control_fused_kernel<<<batch, kFusedCtl, 0, st>>>(vc, seed, batch_index, batch, params_in,
-                                                    params_out, cb, hdr);
 }
 
 size_t plain_workspace_bytes(const VoiceConst& vc, int batch) {
