@@ -29,7 +29,7 @@
 // integers (an FP64 scan waits on the narrow FP64 pipe), and an interval's 21
 // sums are added up over 8 lanes, not 32. Kernels of the plain form's modules,
 // a warp per interval and a scan kernel that handed FP64 point adjoints on took
-// 110.6 us; now 79.2 us (the three under a profiler: 20, 33 and 30).
+// 110.6 us; now 77.3 us (the three under a profiler: 20, 33 and 30).
 
 #include "control_ff.cuh"
 #include "internal.h"
@@ -248,6 +248,8 @@ __global__ void __launch_bounds__(kCT) bwd_recompute(const __grid_constant__ Voi
 // l its samples 16 l .. 16 l + 15, from the last to the first, so that the sum of
 // d/d(phase) over later samples is at hand: over the lane's own it runs along,
 // over the later lanes' it enters the moments afterwards (they are linear in it).
+// Six blocks an SM (80 registers): issue is at half its rate with five, waiting
+// for the sine unit; 79.3 -> 77.3 us. With eight the accumulators spill: 79.7.
 // ---------------------------------------------------------------------------
 constexpr int kST = 128;
 constexpr int kSI = kST / 8;  // intervals per block
@@ -276,10 +278,10 @@ __device__ __forceinline__ void vco_quad_and_inc(const SegVco& s, int j0, float 
   }
 }
 
-__global__ void __launch_bounds__(kST) bwd_samples(const __grid_constant__ VoiceConst vc,
-                                                   uint64_t seed, uint64_t batch_index, int batch,
-                                                   const float* __restrict__ grad_audio,
-                                                   const AdjBuffers b, ScratchHeader* hdr) {
+__global__ void __launch_bounds__(kST, 6) bwd_samples(const __grid_constant__ VoiceConst vc,
+                                                      uint64_t seed, uint64_t batch_index, int batch,
+                                                      const float* __restrict__ grad_audio,
+                                                      const AdjBuffers b, ScratchHeader* hdr) {
   const int lane = threadIdx.x & 31, l8 = lane & 7;
   const int v = blockIdx.y;
   const int K = vc.K, P = K + 1, R = vc.R;
