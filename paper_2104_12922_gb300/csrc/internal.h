@@ -96,6 +96,7 @@ struct PeakNormArgs {
   float threshold;     // voices with peak >= threshold (and > 0) are scaled to peak 1
   float* peak_out;     // [batch] peak |sample| of each voice as rendered, nullable
   int32_t* silent_out; // [batch] 1 where the voice was left as rendered, nullable
+  int scale_ctas;      // CTAs that take scaling items once the tiles are out (set at the launch)
 };
 constexpr int kNormChunkSamples = 8192;  // samples per normalisation work item
 

@@ -52,7 +52,8 @@ struct PhiloxNoise {
   uint32_t z2;            // round 2: low(M0 word 0) ^ key word 1
   uint32_t x3;            // round 3: low(M1 z1) ^ key word 0
   uint32_t z3;            // round 3: key word 1
-  uint32_t kx[7], ky[7];  // keys of rounds 4..10
+  uint32_t k[14];         // keys of rounds 4..10 (word 0, word 1 of each)
+  uint32_t pad;
 };
 
 SYNTH_PHILOX_HD PhiloxNoise philox_noise_setup(uint32_t c0, uint32_t c1, uint32_t c3, uint32_t k0,
@@ -76,9 +77,10 @@ SYNTH_PHILOX_HD PhiloxNoise philox_noise_setup(uint32_t c0, uint32_t c1, uint32_
   for (int r = 0; r < 7; ++r) {
     k0 += kPhiloxW0;
     k1 += kPhiloxW1;
-    p.kx[r] = k0;
-    p.ky[r] = k1;
+    p.k[2 * r] = k0;
+    p.k[2 * r + 1] = k1;
   }
+  p.pad = 0;
   return p;
 }
 
@@ -106,9 +108,9 @@ SYNTH_PHILOX_HD void philox_noise(const PhiloxNoise& p, uint32_t q, uint32_t out
     l0 = kPhiloxM0 * x;
     h1 = philox_mulhi(kPhiloxM1, z);
     l1 = kPhiloxM1 * z;
-    x = h1 ^ y ^ p.kx[r];
+    x = h1 ^ y ^ p.k[2 * r];
     y = l1;
-    z = h0 ^ w ^ p.ky[r];
+    z = h0 ^ w ^ p.k[2 * r + 1];
     w = l0;
   }
   out[0] = x;
@@ -116,5 +118,49 @@ SYNTH_PHILOX_HD void philox_noise(const PhiloxNoise& p, uint32_t q, uint32_t out
   out[2] = z;
   out[3] = w;
 }
+
+#if defined(__CUDACC__)
+// The same with the fixed parts in shared memory (16-byte aligned), loaded
+// where they are used, four words at a time: held in registers, or left to the
+// compiler to hoist, they spill the render's audio loop.
+__device__ __forceinline__ uint4 philox_noise_shared(const PhiloxNoise* p, uint32_t q) {
+  const uint32_t at = (uint32_t)__cvta_generic_to_shared(p);
+  uint32_t f[4];
+  auto fixed = [&](int i) {
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(f[0]), "=r"(f[1]), "=r"(f[2]), "=r"(f[3])
+                 : "r"(at + 16 * i));
+  };
+  auto product = [](uint32_t m, uint32_t a, uint32_t& hi, uint32_t& lo) {
+    hi = __umulhi(m, a);
+    lo = m * a;
+  };
+  fixed(0);
+  uint32_t h0, l0, h1, l1, x, y, z, w;
+  product(kPhiloxM1, q, h1, l1);
+  product(kPhiloxM0, h1 ^ f[0], h0, w);
+  x = l1 ^ f[1];
+  z = h0 ^ f[2];
+  product(kPhiloxM0, x, h0, l0);
+  product(kPhiloxM1, z, h1, l1);
+  x = h1 ^ f[3];
+  y = l1;
+  fixed(1);
+  z = h0 ^ w ^ f[0];
+  w = l0;
+#pragma unroll
+  for (int r = 0; r < 7; ++r) {
+    product(kPhiloxM0, x, h0, l0);
+    product(kPhiloxM1, z, h1, l1);
+    // word 5 + 2 r of the struct, then 6 + 2 r
+    x = h1 ^ y ^ f[(1 + 2 * r) & 3];
+    y = l1;
+    if ((2 + 2 * r) % 4 == 0) fixed(1 + (2 + 2 * r) / 4);
+    z = h0 ^ w ^ f[(2 + 2 * r) & 3];
+    w = l0;
+  }
+  return make_uint4(x, y, z, w);
+}
+#endif
 
 }  // namespace synth

@@ -32,6 +32,7 @@
 // FP64 arithmetic runs. Consecutive launches on a stream may overlap (see
 // release_next_launch and the launch record at the end of this file).
 
+#include <climits>
 #include <mutex>
 #include <unordered_map>
 
@@ -76,6 +77,7 @@ struct __align__(16) VoiceSetupRecord {
 
 struct __align__(16) Smem {
   FFTables T;
+  PhiloxNoise noise;         // peak variant: what the voice fixes of its noise draws
   union {
     ff env[6][P];            // the 6 ADSRs at the control points (steps 2-3)
     struct {
@@ -261,8 +263,8 @@ __device__ __noinline__ void normalize_chunk(Smem& s, float* __restrict__ audio,
 }
 
 // Programmatic dependent launch. When a CTA takes a render tile that is
-// likely its last (fewer items remain after it than the grid has CTAs), and
-// after a scaling item that is, it waits for the previous grid on the stream
+// likely its last (fewer tiles remain after it than the grid has CTAs), and
+// at a scaling item if it has not, it waits for the previous grid on the stream
 // to complete (a no-op unless this launch may overlap it) and then releases
 // the next launch on the stream: when every CTA has done so, the next
 // launch's CTAs start in the SM slots that this launch's last wave leaves
@@ -304,14 +306,16 @@ __global__ void __launch_bounds__(NT, kCtasPerSm) render_fused_kernel(
   const float invR = 1.0f / (float)R;
   load_tables(s.T, vc.T);
   if (tid == 0) s.epoch = *(volatile unsigned int*)&hdr->epoch;
-  // all work items of the launch: render tiles, then (peak variant) scaling chunks
-  const int total_items =
-      total_tiles + (kPeak ? (int)((N + kNormChunkSamples - 1) / kNormChunkSamples) * batch : 0);
   bool released = false;
 
   for (;;) {
     if (tid == 0) {
-      const int tc = (int)atomicAdd(&hdr->work, 1u);
+      // peak variant: once the render tiles are out, CTAs past the first
+      // norm.scale_ctas leave the scaling to those (a tile claimed in between,
+      // or an item, is still done)
+      const bool leave = kPeak && (int)blockIdx.x >= norm.scale_ctas &&
+                         *(volatile unsigned int*)&hdr->work >= (unsigned int)total_tiles;
+      const int tc = leave ? INT_MAX : (int)atomicAdd(&hdr->work, 1u);
       s.tile = tc;
       // a later window of a voice whose first window has published its set-up
       int ready = 0;
@@ -330,14 +334,14 @@ __global__ void __launch_bounds__(NT, kCtasPerSm) render_fused_kernel(
       if (!kPeak) { release_next_launch(released); break; }
       const int chunks = (int)((N + kNormChunkSamples - 1) / kNormChunkSamples);
       const int j = t - total_tiles;
-      if (j >= chunks * batch) { release_next_launch(released); break; }
+      release_next_launch(released);
+      if (j >= chunks * batch) break;
       if (!in_bounds(hdr, j / chunks, batch)) continue;
       normalize_chunk(s, audio, N, tiles + (size_t)(j / chunks) * n_windows, n_windows,
                       j / chunks, j % chunks, vec_ok, norm, hdr, s.epoch);
-      if (t + (int)gridDim.x >= total_items) release_next_launch(released);
       continue;
     }
-    if (!kSplit && t + (int)gridDim.x >= total_items)
+    if (!kSplit && t + (int)gridDim.x >= total_tiles)
       release_next_launch(released);  // likely the last tile
     const int v = t % batch, w = t / batch;
     // the tile's voice and window address its set-up, tile and output records
@@ -495,6 +499,8 @@ __global__ void __launch_bounds__(NT, kCtasPerSm) render_fused_kernel(
     }
 
     if (kSplit) release_next_launch(released);
+    if (kPeak && tid == NT - 1)  // a thread without an interval
+      s.noise = philox_noise_setup((uint32_t)g, (uint32_t)(g >> 32), kStreamNoise, key.x, key.y);
 
     // ---- 4. VCO phase over each control interval, scanned -----------------
     ff tot[2] = {ff_make(0.f), ff_make(0.f)};
@@ -627,13 +633,13 @@ __global__ void __launch_bounds__(NT, kCtasPerSm) render_fused_kernel(
         }
       };
       // the noise generator's key schedule and the products the voice fixes,
-      // once per tile (the peak variant keeps the wide-product form)
+      // once per tile (the peak variant: from shared memory)
       const PhiloxNoise pn =
           philox_noise_setup((uint32_t)g, (uint32_t)(g >> 32), kStreamNoise, key.x, key.y);
       auto noise_quad = [&](int rel0) {
         const uint32_t q = (uint32_t)((s_tile + rel0) >> 2);
         if constexpr (kPeak) {
-          return philox4x32_10_wide(make_uint4((uint32_t)g, (uint32_t)(g >> 32), q, kStreamNoise), key);
+          return philox_noise_shared(&s.noise, q);
         } else {
           uint32_t o[4];
           philox_noise(pn, q, o);
@@ -781,10 +787,13 @@ __global__ void __launch_bounds__(NT, kCtasPerSm) render_fused_kernel(
           const float4 A = s.ampv[si], D = s.aslope[si];
           const int jq = j0 + 4 * q;
           const int off = off0 + 4 * q;
-          const uint4 nc =
-              make_uint4((uint32_t)g, (uint32_t)(g >> 32), q_t + (uint32_t)(off >> 2), kStreamNoise);
-          // the peak variant: the wide-product form, which leaves it no spills
-          const uint4 nz = kPeak ? philox4x32_10_wide(nc, key) : philox4x32_10(nc, key);
+          const uint32_t qn = q_t + (uint32_t)(off >> 2);
+          // the peak variant: the fixed parts from shared memory, which leaves it
+          // fewer spills than products held or formed anew (122 -> 116 us for 128 x
+          // 4 s); the other variant has none and is 1% faster with the plain rounds
+          const uint4 nz = kPeak ? philox_noise_shared(&s.noise, qn)
+                                 : philox4x32_10(make_uint4((uint32_t)g, (uint32_t)(g >> 32), qn,
+                                                            kStreamNoise), key);
           const uint32_t nw[4] = {nz.x, nz.y, nz.z, nz.w};
           // amplitudes at the quad's first sample, then one step of the slope per sample
           const float fj0 = (float)jq;
@@ -931,6 +940,7 @@ cudaError_t launch_render_fused(const VoiceConst& vc, uint64_t seed, uint64_t fi
                                 void* voice_setups) {
   const int n_windows = windows_per_voice(vc.K);
   const int total = batch * n_windows;
+  const int full_grid = grid;
   // a launch whose tiles are all resident at once; where they leave SMs empty,
   // each tile goes to as many CTAs as give every SM one (a second CTA on an SM
   // slows the first one's control steps by more than it saves), at most
@@ -940,7 +950,14 @@ cudaError_t launch_render_fused(const VoiceConst& vc, uint64_t seed, uint64_t fi
   parts = parts < 1 ? 1 : parts < kMaxParts ? parts : kMaxParts;
   if (parts > 1) voice_setups = nullptr;  // no window starts after another has finished
   grid = grid < total * parts ? grid : total * parts;
-  const PeakNormArgs nz = norm ? *norm : PeakNormArgs{0.f, nullptr, nullptr};
+  PeakNormArgs nz = norm ? *norm : PeakNormArgs{0.f, nullptr, nullptr, 0};
+  // Half the resident CTAs scale: that is bound by memory, not by CTAs, and the
+  // others make room for the next launch, whose control steps and audio run
+  // beside it. 128 x 4 s, launches in a row, 100 / 85 / 70 / 60 / 50 / 40 / 30% of
+  // the CTAs: 111.7 / 108.6 / 101.6 / 97.3 / 94.8 / 99.3 / 111.2 us; at 48 kHz 139.6
+  // / 136.9 / 132.0 / 129.6 / 124.2 / 128.5 / 137.2. Where the next launch may not
+  // overlap this one, 100 / 50 / 30%: 118.9 / 120.7 / 135.0.
+  nz.scale_ctas = full_grid / 2;
   if (sub_batch <= 0) sub_batch = batch;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);

@@ -242,7 +242,7 @@ synth_status synth_render_normalized(synth_handle h, uint64_t seed, uint64_t bat
   if (!audio_dev) return SYNTH_ERR_ARG;
   ScratchHeader* hdr = take_overlap_slot(h);
   TileState* tiles = reinterpret_cast<TileState*>(hdr + 1);
-  const PeakNormArgs norm{threshold, peak_out_dev, silent_out_dev};
+  const PeakNormArgs norm{threshold, peak_out_dev, silent_out_dev, 0};
   return check_cuda(launch_render_fused(h->vc, seed, batch_index * (uint64_t)batch, 0, batch,
                                         params_in_dev, audio_dev, params_out_dev, hdr, tiles,
                                         h->fused_grid, static_cast<cudaStream_t>(stream), &norm,
