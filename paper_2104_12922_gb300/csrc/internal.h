@@ -29,8 +29,9 @@ static_assert(sizeof(ScratchHeader) == 256, "header is one 256-byte block");
 // 64-bit fixed-point phase, or the bits of a float in the FP32-carry mode.
 struct TileState {
   unsigned int flag[2];  // (epoch << 2) | 1 once agg[chain] of this launch is published
-  unsigned int done;      // (epoch << 2) | 3 once the tile's audio is written (peak variant)
-  unsigned int peak;      // the bits of the tile's largest |sample| (peak variant)
+  // peak variant: (epoch << 4) | CTAs that have written their part of the tile's
+  // audio, and above it the bits of the largest |sample| they wrote
+  unsigned long long done_peak;
   unsigned long long agg[2][2];
 };
 static_assert(sizeof(TileState) == 48, "tile state layout");

@@ -171,9 +171,12 @@ __device__ __forceinline__ void block_scan2_f32(float& a, float& b, float (*buf)
   tot1 = tb;
 }
 
-// The tile's peak (a block maximum of the threads' largest |sample|),
-// published in its tile record behind a done flag once every thread's
-// stores are visible at device scope.
+// This CTA's part of a tile's peak (a block maximum of the threads' largest
+// |sample|), joined to the other parts' in the tile's record together with their
+// count, once every thread's stores are visible at device scope. A record of an
+// earlier launch counts as empty.
+__device__ __forceinline__ unsigned int tile_done_tag(unsigned int epoch) { return (epoch & 0x0fffffffu) << 4; }
+template <bool kSplit>
 __device__ __forceinline__ void publish_tile_peak(Smem& s, TileState* me, float vmax,
                                                   unsigned int epoch) {
   const int tid = threadIdx.x;
@@ -186,9 +189,20 @@ __device__ __forceinline__ void publish_tile_peak(Smem& s, TileState* me, float 
     float m = s.warp_max[0];
 #pragma unroll
     for (int i = 1; i < kWarps; ++i) m = fmaxf(m, s.warp_max[i]);
-    me->peak = __float_as_uint(m);
-    cuda::atomic_ref<unsigned int, cuda::thread_scope_device> f(me->done);
-    f.store(((epoch & 0x3fffffffu) << 2) | 3u, cuda::memory_order_release);
+    // bits of non-negative floats order as integers
+    const unsigned int tag = tile_done_tag(epoch);
+    cuda::atomic_ref<u64, cuda::thread_scope_device> f(me->done_peak);
+    if (kSplit) {
+      u64 old = f.load(cuda::memory_order_relaxed), next;
+      do {
+        const bool own = ((unsigned int)old & ~15u) == tag && ((unsigned int)old & 15u) != 0;
+        const unsigned int count = own ? (unsigned int)old & 15u : 0u;
+        const unsigned int best = own ? max((unsigned int)(old >> 32), __float_as_uint(m)) : __float_as_uint(m);
+        next = ((u64)best << 32) | tag | (count + 1u);
+      } while (!f.compare_exchange_weak(old, next, cuda::memory_order_acq_rel, cuda::memory_order_relaxed));
+    } else {
+      f.store(((u64)__float_as_uint(m) << 32) | tag | 1u, cuda::memory_order_release);
+    }
   }
 }
 
@@ -202,15 +216,17 @@ __device__ __forceinline__ void publish_tile_peak(Smem& s, TileState* me, float 
 __device__ __noinline__ void normalize_chunk(Smem& s, float* __restrict__ audio, int64_t N,
                                              TileState* vt, int n_windows, int v, int c,
                                              bool vec_ok, const PeakNormArgs& norm,
-                                             ScratchHeader* hdr, unsigned int epoch) {
+                                             ScratchHeader* hdr, unsigned int epoch, int parts) {
   const int tid = threadIdx.x;
-  const unsigned int tag = ((epoch & 0x3fffffffu) << 2) | 3u;
+  const unsigned int tag = tile_done_tag(epoch) | (unsigned int)parts;
   float m = 0.f;
   for (int w = tid; w < n_windows; w += NT) {
-    cuda::atomic_ref<unsigned int, cuda::thread_scope_device> f(vt[w].done);
+    cuda::atomic_ref<u64, cuda::thread_scope_device> f(vt[w].done_peak);
     bool ready = false;
+    u64 got = 0;
     for (int spins = 0; spins < kLookbackSpinLimit; ++spins) {
-      if (f.load(cuda::memory_order_acquire) == tag) { ready = true; break; }
+      got = f.load(cuda::memory_order_acquire);
+      if ((unsigned int)got == tag) { ready = true; break; }
       if (*(volatile unsigned int*)&hdr->error) break;
       __nanosleep(128);
     }
@@ -218,7 +234,7 @@ __device__ __noinline__ void normalize_chunk(Smem& s, float* __restrict__ audio,
       atomicOr(&hdr->error, kErrTileWaitTimeout);
       break;
     }
-    m = fmaxf(m, __uint_as_float(__ldcg(&vt[w].peak)));
+    m = fmaxf(m, __uint_as_float((unsigned int)(got >> 32)));
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -288,7 +304,10 @@ __device__ __forceinline__ void release_next_launch(bool& released) {
 // every tile of this one from starting, where with it in the middle two
 // launches in a row overlap. One 4 s voice a launch, launches in a row: 28.0 ->
 // 11.7 us (alone 32.4 -> 24.3), 8 voices 31.2 -> 17.7, 16: 35.2 -> 27.3, 32: 44.1
-// -> 35.2, 64: 58.0 -> 42.6, 80: 62.4 -> 51.7.
+// -> 35.2, 64: 58.0 -> 42.6, 80: 62.4 -> 51.7. Normalised, where the parts of a tile
+// join their peaks in its record: 1 voice 42.4 -> 22.3, 5: 52.4 -> 27.4, 40: 54.3 ->
+// 45.3, 84: 81.6 -> 72.1; where launches may not overlap, 47.7 -> 35.3, 56.9 -> 39.6,
+// 57.5 -> 57.4, 88.7 -> 87.4.
 template <bool kCarryF32, bool kPeak, bool kGenR, bool kSplit>
 __global__ void __launch_bounds__(NT, kCtasPerSm) render_fused_kernel(
     const __grid_constant__ VoiceConst vc, uint64_t seed, uint64_t first, int split, int batch,
@@ -298,7 +317,7 @@ __global__ void __launch_bounds__(NT, kCtasPerSm) render_fused_kernel(
   __shared__ Smem s;
   const int tid = threadIdx.x;
   const int total_tiles = batch * n_windows;
-  static_assert(!kSplit || !kPeak, "a tile's peak is one CTA's");
+  static_assert(kMaxParts < 16, "the parts of a tile are counted in 4 bits");
   const int R = vc.R, K = vc.K;
   const int64_t N = vc.n_samples;
   const int qps = R >> 2;             // quads per control interval
@@ -314,7 +333,7 @@ __global__ void __launch_bounds__(NT, kCtasPerSm) render_fused_kernel(
       // norm.scale_ctas leave the scaling to those (a tile claimed in between,
       // or an item, is still done)
       const bool leave = kPeak && (int)blockIdx.x >= norm.scale_ctas &&
-                         *(volatile unsigned int*)&hdr->work >= (unsigned int)total_tiles;
+                         *(volatile unsigned int*)&hdr->work >= (unsigned int)(total_tiles * parts);
       const int tc = leave ? INT_MAX : (int)atomicAdd(&hdr->work, 1u);
       s.tile = tc;
       // a later window of a voice whose first window has published its set-up
@@ -326,19 +345,20 @@ __global__ void __launch_bounds__(NT, kCtasPerSm) render_fused_kernel(
       s.setup_ready = ready;
     }
     __syncthreads();  // also: the previous tile's audio is done with the shared buffers
+    const bool is_tile = s.tile < total_tiles * (kSplit ? parts : 1);
     const int t = kSplit ? s.tile / parts : s.tile;
     const int part = kSplit ? s.tile - t * parts : 0;
-    if (t >= total_tiles) {
+    if (!is_tile) {
       // peak variant: the scaling chunks follow the render tiles, voice by
       // voice (window-major tiles finish their voices in that order)
       if (!kPeak) { release_next_launch(released); break; }
       const int chunks = (int)((N + kNormChunkSamples - 1) / kNormChunkSamples);
-      const int j = t - total_tiles;
+      const int j = s.tile - total_tiles * (kSplit ? parts : 1);
       release_next_launch(released);
       if (j >= chunks * batch) break;
       if (!in_bounds(hdr, j / chunks, batch)) continue;
       normalize_chunk(s, audio, N, tiles + (size_t)(j / chunks) * n_windows, n_windows,
-                      j / chunks, j % chunks, vec_ok, norm, hdr, s.epoch);
+                      j / chunks, j % chunks, vec_ok, norm, hdr, s.epoch, parts);
       continue;
     }
     if (!kSplit && t + (int)gridDim.x >= total_tiles)
@@ -758,7 +778,7 @@ __global__ void __launch_bounds__(NT, kCtasPerSm) render_fused_kernel(
           }
         }
       }
-      if (kPeak) publish_tile_peak(s, vt + w, vmax, epoch);
+      if (kPeak) publish_tile_peak<kSplit>(s, vt + w, vmax, epoch);
     } else {
       const int64_t t0 = (int64_t)k0 * R;                     // first sample of the tile
       float* out_t = audio + (size_t)v * (size_t)N + (size_t)t0;
@@ -873,7 +893,7 @@ __global__ void __launch_bounds__(NT, kCtasPerSm) render_fused_kernel(
           }
         }
       }
-      if (kPeak) publish_tile_peak(s, vt + w, vmax, epoch);
+      if (kPeak) publish_tile_peak<kSplit>(s, vt + w, vmax, epoch);
     }
   }
   persistent_finish(hdr);
@@ -945,7 +965,7 @@ cudaError_t launch_render_fused(const VoiceConst& vc, uint64_t seed, uint64_t fi
   // each tile goes to as many CTAs as give every SM one (a second CTA on an SM
   // slows the first one's control steps by more than it saves), at most
   // kMaxParts (beyond, the copies of the control steps no longer pay)
-  const bool shared = !norm && !vc.carry_fp32 && total <= grid;
+  const bool shared = !vc.carry_fp32 && total <= grid;
   int parts = shared ? grid / kCtasPerSm / total : 1;
   parts = parts < 1 ? 1 : parts < kMaxParts ? parts : kMaxParts;
   if (parts > 1) voice_setups = nullptr;  // no window starts after another has finished
@@ -990,14 +1010,16 @@ cudaError_t launch_render_fused(const VoiceConst& vc, uint64_t seed, uint64_t fi
                          n_windows, nz, seed_step, sub_batch, setups, parts
   cudaError_t e;
   if (vc.general_r) {  // fractional R (never with FP32 carries)
-    if (norm) e = cudaLaunchKernelEx(&cfg, render_fused_kernel<false, true, true, false>, SYNTH_FUSED_ARGS);
+    if (norm && shared) e = cudaLaunchKernelEx(&cfg, render_fused_kernel<false, true, true, true>, SYNTH_FUSED_ARGS);
+    else if (norm) e = cudaLaunchKernelEx(&cfg, render_fused_kernel<false, true, true, false>, SYNTH_FUSED_ARGS);
     else if (shared) e = cudaLaunchKernelEx(&cfg, render_fused_kernel<false, false, true, true>, SYNTH_FUSED_ARGS);
     else e = cudaLaunchKernelEx(&cfg, render_fused_kernel<false, false, true, false>, SYNTH_FUSED_ARGS);
   } else if (vc.carry_fp32) {
     if (norm) e = cudaLaunchKernelEx(&cfg, render_fused_kernel<true, true, false, false>, SYNTH_FUSED_ARGS);
     else e = cudaLaunchKernelEx(&cfg, render_fused_kernel<true, false, false, false>, SYNTH_FUSED_ARGS);
   } else {
-    if (norm) e = cudaLaunchKernelEx(&cfg, render_fused_kernel<false, true, false, false>, SYNTH_FUSED_ARGS);
+    if (norm && shared) e = cudaLaunchKernelEx(&cfg, render_fused_kernel<false, true, false, true>, SYNTH_FUSED_ARGS);
+    else if (norm) e = cudaLaunchKernelEx(&cfg, render_fused_kernel<false, true, false, false>, SYNTH_FUSED_ARGS);
     else if (shared) e = cudaLaunchKernelEx(&cfg, render_fused_kernel<false, false, false, true>, SYNTH_FUSED_ARGS);
     else e = cudaLaunchKernelEx(&cfg, render_fused_kernel<false, false, false, false>, SYNTH_FUSED_ARGS);
   }
