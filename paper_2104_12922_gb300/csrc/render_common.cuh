@@ -108,10 +108,7 @@ __device__ __forceinline__ float vco_phase_at(const SegVco& s, int jc, int j) {
   return p - rintf(p);
 }
 
-// kRolled: a quad that straddles the piece boundary is evaluated by a rolled
-// loop (one copy of the per-sample code: a smaller loop body where such quads
-// are rare, i.e. whenever quads align with the intervals); unrolled otherwise.
-template <bool kWrap = true, bool kRolled = true>
+template <bool kWrap = true>
 __device__ __forceinline__ void vco_quad(const SegVco& s, int j0, float ph[4]) {
   const int jc = s.jc_flags & 0xffff;
   if (j0 + 3 < jc || j0 >= jc) {
@@ -134,7 +131,7 @@ __device__ __forceinline__ void vco_quad(const SegVco& s, int j0, float ph[4]) {
     ph[1] = kWrap ? p1 - rintf(p1) : p1;
     ph[2] = kWrap ? p2 - rintf(p2) : p2;
     ph[3] = kWrap ? p3 - rintf(p3) : p3;
-  } else if (kRolled) {  // the quad straddles the piece boundary: one rolled loop
+  } else {  // the quad straddles the piece boundary: one rolled loop, since few do
 #pragma unroll 1
     for (int i = 0; i < 4; ++i) {
       const float w = vco_phase_at(s, jc, j0 + i);
@@ -143,9 +140,6 @@ __device__ __forceinline__ void vco_quad(const SegVco& s, int j0, float ph[4]) {
       if (i == 2) ph[2] = w;
       if (i == 3) ph[3] = w;
     }
-  } else {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) ph[i] = vco_phase_at(s, jc, j0 + i);
   }
 }
 
@@ -162,15 +156,15 @@ struct VcoRun {
   float base, g;
 };
 
-// Starts a run at sample j0 of the interval for `len` samples; false when
-// the samples straddle the piece boundary jc, or lie in a piece of another
-// kind than the interval's steps describe (a linear piece beside a geometric
-// one): the caller then evaluates each quad on its own. The start is the
-// quad formula of vco_quad.
-__device__ __forceinline__ bool vco_run_start(const SegVco& s, int j0, int len, VcoRun& r) {
+// Starts a run at sample j0 of the interval (negative for a quad that straddles
+// the interval's start) whose samples lo .. hi the caller uses; false when those
+// straddle the piece boundary jc, or lie in a piece of another kind than the
+// interval's steps describe (a linear piece beside a geometric one): the caller
+// then evaluates each quad on its own. The start is the quad formula of vco_quad.
+__device__ __forceinline__ bool vco_run_start(const SegVco& s, int j0, int lo, int hi, VcoRun& r) {
   const int jc = s.jc_flags & 0xffff;
-  if (!(j0 + len - 1 < jc || j0 >= jc)) return false;
-  const bool in_b = j0 >= jc;
+  if (!(hi < jc || lo >= jc)) return false;
+  const bool in_b = lo >= jc;
   const float L = in_b ? s.LB : 0.f;
   const float c = in_b ? s.cB : s.cA;
   const bool lin = (s.jc_flags >> (in_b ? 17 : 16)) & 1;

@@ -85,18 +85,19 @@ struct __align__(16) Smem {
       union {
         float4 aslope[TI];   // R a multiple of 4: amplitude change per sample over each
                              // interval, (ampv[k + 1] - ampv[k]) / R
-        struct {
-          int sst[P];        // fractional R: first sample of each interval (tile-relative),
+        int sst[P];          // general R: first sample of each interval (tile-relative),
                              // sst[nseg] = the tile's sample count
-          float u0f[TI];     // fractional R: fraction of each interval's first sample
-        };
       };
     };
   };
   float4 sq[TI];             // square-saw constants per interval: k2, c1, c2 (square_saw_sc)
   float4 ampv[P];            // gain x amplitude at the control points: sine, square-saw (gain
-                             // folded into sq), noise
-  ff m[2][P];                // VCO pitch (midi) at the control points
+                             // folded into sq), noise; general R, from step 5 on: at each
+                             // interval's first sample
+  union {
+    ff m[2][P];              // VCO pitch (midi) at the control points
+    float4 aslope_g[TI];     // general R, step 5: aslope
+  };
   ff y[kNumParams];          // human-range parameters
   VoiceSetup vs;
   float u[80];
@@ -524,6 +525,7 @@ __global__ void __launch_bounds__(NT, kCtasPerSm) render_fused_kernel(
 
     // ---- 4. VCO phase over each control interval, scanned -----------------
     ff tot[2] = {ff_make(0.f), ff_make(0.f)};
+    float4 a_first = make_float4(0.f, 0.f, 0.f, 0.f), a_slope = a_first;  // general R
     // the tile's first sample: interval k starts at sample ceil(k a / b)
     const int64_t s_tile =
         kGenR ? ((int64_t)k0 * vc.rate_a + vc.rate_b - 1) / vc.rate_b : (int64_t)k0 * R;
@@ -537,8 +539,13 @@ __global__ void __launch_bounds__(NT, kCtasPerSm) render_fused_kernel(
         // fraction of the way from point k to point k + 1: (s_k b - k a) / a
         const ff u0 = ff_mul_f(vc.inv_a, (float)(sk * vc.rate_b - k * vc.rate_a));
         s.sst[tid] = (int)(sk - s_tile);
-        s.u0f[tid] = ff_to_float(u0);
         if (tid == nseg - 1) s.sst[nseg] = (int)(sk1 - s_tile);
+        {  // the amplitudes at the interval's first sample and their change per sample
+          const float4 a = s.ampv[tid], b = s.ampv[tid + 1];
+          const float u = ff_to_float(u0), ir = ff_to_float(vc.inv_R);
+          a_first = make_float4(fmaf(u, b.x - a.x, a.x), fmaf(u, b.y - a.y, a.y), fmaf(u, b.z - a.z, a.z), 0.f);
+          a_slope = make_float4((b.x - a.x) * ir, (b.y - a.y) * ir, (b.z - a.z) * ir, 0.f);
+        }
         // the pitch at the interval's first sample, and the end point that
         // keeps the slope (m_(k+1) - m_k) / R per sample
 #pragma unroll 1
@@ -611,6 +618,10 @@ __global__ void __launch_bounds__(NT, kCtasPerSm) render_fused_kernel(
         s.seg[1][tid].phase0 = carry_wrap(fix64_to_float(s.vs.vco_p0[1]) + s.prefix_f[1] + c1);
       }
     }
+    if (kGenR && tid < nseg) {  // the points were last read before the scan's barrier
+      s.ampv[tid] = a_first;
+      s.aslope_g[tid] = a_slope;
+    }
     __syncthreads();
 
     // ---- 5. audio ----------------------------------------------------------
@@ -618,129 +629,48 @@ __global__ void __launch_bounds__(NT, kCtasPerSm) render_fused_kernel(
     const int seg0 = kSplit ? nseg * part / parts : 0;
     const int seg1 = kSplit ? nseg * (part + 1) / parts : nseg;
     if constexpr (kGenR) {
-      // fractional R: quads of the voice's own 4-sample grid. A work item is
-      // (interval, chunk): the quad that straddles the interval's start is
-      // evaluated on its own (each sample in the interval whose start it has
-      // passed; a quad meets at most two intervals since R >= 4), the quads
-      // inside the interval in runs of kGenG, their VCO phases stepped from
-      // quad to quad as on the default path. The tile writes only its own
-      // samples.
-      const int n_t = s.sst[nseg];
+      // general R: quads of the voice's own 4-sample grid, which the noise
+      // generator counts. An interval takes every quad it has a sample in, in
+      // runs of up to kGenG (a work item); of a quad that straddles its start or
+      // end it writes its own samples, the neighbour the others. That evaluates
+      // such a quad twice; once, in a loop of its own that found its interval and
+      // formed both intervals' phases, it cost more, and the runs, bounded by two
+      // quads more than an interval has, left a third of the threads idle at 16
+      // kHz. 128 x 4 s: 16 kHz 78.6 -> 61.2 us, 22.05 kHz 77.8 -> 70.4, 48 kHz 101.3 ->
+      // 92.5; six such batches a launch at 16 kHz 407 -> 290; one voice 16.4 -> 12.6.
+      constexpr int kGenG = 5;
       float* out_v = audio + (size_t)v * (size_t)N;
-      const float invRg = ff_to_float(vc.inv_R);
       float vmax = 0.f;
-      // a quad's four samples at tile-relative sample rel0: 16-byte stores
-      // inside the tile, else the samples in [0, n_t) one by one
-      auto store_quad = [&](int rel0, const float out4[4]) {
-        const int64_t n0 = s_tile + rel0;
-        if (vec_ok && rel0 >= 0 && rel0 + 3 < n_t) {
-          if (!in_bounds(hdr, n0, N) || !in_bounds(hdr, n0 + 3, N)) return;
-          if (kPeak) {
-            *reinterpret_cast<float4*>(out_v + n0) = make_float4(out4[0], out4[1], out4[2], out4[3]);
-            vmax = fmaxf(fmaxf(vmax, fmaxf(fabsf(out4[0]), fabsf(out4[1]))),
-                         fmaxf(fabsf(out4[2]), fabsf(out4[3])));
-          } else {
-            __stcs(reinterpret_cast<float4*>(out_v + n0),
-                   make_float4(out4[0], out4[1], out4[2], out4[3]));
-          }
-        } else {
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            if (rel0 + i >= 0 && rel0 + i < n_t && in_bounds(hdr, n0 + i, N)) {
-              out_v[n0 + i] = out4[i];
-              if (kPeak) vmax = fmaxf(vmax, fabsf(out4[i]));
-            }
-        }
-      };
+      const int full_q = (vc.R + 2) / 4 + 1;            // bound on an interval's quads
+      const int cpi = (full_q + kGenG - 1) / kGenG;     // runs per interval
+      const int G = (full_q + cpi - 1) / cpi;           // quads per run
       // the noise generator's key schedule and the products the voice fixes,
       // once per tile (the peak variant: from shared memory)
       const PhiloxNoise pn =
           philox_noise_setup((uint32_t)g, (uint32_t)(g >> 32), kStreamNoise, key.x, key.y);
-      auto noise_quad = [&](int rel0) {
-        const uint32_t q = (uint32_t)((s_tile + rel0) >> 2);
-        if constexpr (kPeak) {
-          return philox_noise_shared(&s.noise, q);
-        } else {
-          uint32_t o[4];
-          philox_noise(pn, q, o);
-          return make_uint4(o[0], o[1], o[2], o[3]);
-        }
-      };
-      // a quad on its own, its interval found from a float estimate
-      auto single_quad = [&](int rel0) {
-        const int r0 = max(rel0, 0);
-        int si = min((int)((float)r0 * invRg), nseg - 1);
-        while (si + 1 < nseg && s.sst[si + 1] <= r0) ++si;
-        while (si > 0 && s.sst[si] > r0) --si;
-        const int b1 = s.sst[si + 1];
-        const bool two = si + 1 < nseg && rel0 + 3 >= b1;
-        float psA[4], pqA[4], psB[4], pqB[4];
-        vco_quad<false, false>(s.seg[0][si], rel0 - s.sst[si], psA);
-        vco_quad<false, false>(s.seg[1][si], rel0 - s.sst[si], pqA);
-        if (two) {
-          vco_quad<false, false>(s.seg[0][si + 1], rel0 - b1, psB);
-          vco_quad<false, false>(s.seg[1][si + 1], rel0 - b1, pqB);
-        }
-        const uint4 nz = noise_quad(rel0);
-        const uint32_t nw[4] = {nz.x, nz.y, nz.z, nz.w};
-        float out4[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int rel = rel0 + i;
-          const bool in_b = two && rel >= b1;
-          const int ii = in_b ? si + 1 : si;
-          const float ps = in_b ? psB[i] : psA[i], pq = in_b ? pqB[i] : pqA[i];
-          const float4 sq = s.sq[ii];
-          const float4 A = s.ampv[ii], Bn = s.ampv[ii + 1];
-          const float fj = fmaf((float)(rel - s.sst[ii]), invRg, s.u0f[ii]);
-          const float x_sin = __sinf(kTwoPiF * ps);
-          float sn, cs;
-          __sincosf(kTwoPiF * pq, &sn, &cs);
-          const float x_sq = square_saw_sc(sn, cs, sq.x, sq.y, sq.z);
-          const float x_nz = fmaf((float)(nw[i] >> 8), 0x1p-23f, -1.f);
-          out4[i] = fmaf(fmaf(fj, Bn.x - A.x, A.x), x_sin,
-                         fmaf(fmaf(fj, Bn.y - A.y, A.y), x_sq, fmaf(fj, Bn.z - A.z, A.z) * x_nz));
-        }
-        store_quad(rel0, out4);
-      };
-      // first the quads that straddle an interval's start (or the tile's
-      // start or end), one loop of their own so that the run loop below
-      // carries none of their state
-      for (int si = seg0 + tid; si < seg1; si += NT) {
-        const int a = s.sst[si], b = s.sst[si + 1];
-        const int f = a + (int)((-(s_tile + a)) & 3);  // first grid quad at or after a
-        const int nf = b - f >= 4 ? (b - f) >> 2 : 0;   // quads wholly inside [a, b)
-        const int tail = f + 4 * nf;
-        const int n_single = (f > a ? 1 : 0) + (si == nseg - 1 && tail < b ? 1 : 0);
-#pragma unroll 1
-        for (int k = 0; k < n_single; ++k) single_quad(k == 0 && f > a ? f - 4 : tail);
-      }
-      // then the whole quads: work items of kGenG quads of one interval
-      constexpr int kGenG = 5;
-      const int full_max = (int)(vc.r_f * 0.25f) + 2;  // bound on an interval's whole quads
-      const int cpi = (full_max + kGenG - 1) / kGenG;   // chunks per interval
       for (int it = seg0 * cpi + tid; it < seg1 * cpi; it += NT) {
         const int si = it / cpi, c = it - si * cpi;
         const int a = s.sst[si], b = s.sst[si + 1];
-        const int f = a + (int)((-(s_tile + a)) & 3);
-        const int nf = b - f >= 4 ? (b - f) >> 2 : 0;
-        const int q0 = c * kGenG, q1 = min(nf, q0 + kGenG);
-        if (q0 >= q1) continue;
+        const int rel_q = a - (int)((s_tile + a) & 3) + 4 * G * c;  // the run's first sample
+        const int nq = min(G, (b - rel_q + 3) >> 2);
+        if (nq <= 0) continue;
         const SegVco& sv0 = s.seg[0][si];
         const SegVco& sv1 = s.seg[1][si];
-        // one whole quad from its VCO phases (radians)
+        // one quad from its VCO phases (radians)
         auto emit = [&](int rel0, const float ps[4], const float pq[4]) {
           const float4 sq = s.sq[si];
-          const float4 A = s.ampv[si], Bn = s.ampv[si + 1];
-          const float u0 = s.u0f[si];
-          // amplitudes: A + (Bn - A) ((rel - a) / R + u0), linear in rel
-          const float dx = (Bn.x - A.x) * invRg, dy = (Bn.y - A.y) * invRg, dz = (Bn.z - A.z) * invRg;
+          const float4 A = s.ampv[si], D = s.aslope_g[si];
+          const uint32_t qn = (uint32_t)((s_tile + rel0) >> 2);
+          uint32_t nw[4];
+          if constexpr (kPeak) {
+            const uint4 nz = philox_noise_shared(&s.noise, qn);
+            nw[0] = nz.x; nw[1] = nz.y; nw[2] = nz.z; nw[3] = nz.w;
+          } else {
+            philox_noise(pn, qn, nw);
+          }
+          // amplitudes at the quad's first sample, then one step of the slope per sample
           const float fj0 = (float)(rel0 - a);
-          const float a0x = fmaf(fj0, dx, fmaf(u0, Bn.x - A.x, A.x));
-          const float a0y = fmaf(fj0, dy, fmaf(u0, Bn.y - A.y, A.y));
-          const float a0z = fmaf(fj0, dz, fmaf(u0, Bn.z - A.z, A.z));
-          const uint4 nz = noise_quad(rel0);
-          const uint32_t nw[4] = {nz.x, nz.y, nz.z, nz.w};
+          const float a0x = fmaf(fj0, D.x, A.x), a0y = fmaf(fj0, D.y, A.y), a0z = fmaf(fj0, D.z, A.z);
           float out4[4];
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
@@ -750,31 +680,50 @@ __global__ void __launch_bounds__(NT, kCtasPerSm) render_fused_kernel(
             const float x_sq = square_saw_sc(sn, cs, sq.x, sq.y, sq.z);
             const float x_nz = fmaf((float)(nw[i] >> 8), 0x1p-23f, -1.f);  // 2u - 1, exact
             const float fi = (float)i;
-            out4[i] = fmaf(fmaf(fi, dx, a0x), x_sin,
-                           fmaf(fmaf(fi, dy, a0y), x_sq, fmaf(fi, dz, a0z) * x_nz));
+            out4[i] = fmaf(fmaf(fi, D.x, a0x), x_sin,
+                           fmaf(fmaf(fi, D.y, a0y), x_sq, fmaf(fi, D.z, a0z) * x_nz));
           }
-          store_quad(rel0, out4);
+          // 16-byte stores inside the interval, else its samples one by one
+          const int64_t n0 = s_tile + rel0;
+          if (vec_ok && rel0 >= a && rel0 + 3 < b &&
+              in_bounds(hdr, n0, N) && in_bounds(hdr, n0 + 3, N)) {
+            const float4 o = make_float4(out4[0], out4[1], out4[2], out4[3]);
+            if (kPeak) {
+              *reinterpret_cast<float4*>(out_v + n0) = o;
+              vmax = fmaxf(fmaxf(vmax, fmaxf(fabsf(o.x), fabsf(o.y))), fmaxf(fabsf(o.z), fabsf(o.w)));
+            } else {
+              __stcs(reinterpret_cast<float4*>(out_v + n0), o);
+            }
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              if (rel0 + i >= a && rel0 + i < b && in_bounds(hdr, n0 + i, N)) {
+                out_v[n0 + i] = out4[i];
+                if (kPeak) vmax = fmaxf(vmax, fabsf(out4[i]));
+              }
+          }
         };
         VcoRun r0, r1;
-        const int j0 = f + 4 * q0 - a;  // the chunk's first sample in its interval
-        if (vco_run_start(sv0, j0, 4 * (q1 - q0), r0) & vco_run_start(sv1, j0, 4 * (q1 - q0), r1)) {
+        // the run's samples in the interval: [lo, hi]
+        const int j0 = rel_q - a, lo = max(j0, 0), hi = min(rel_q + 4 * nq, b) - 1 - a;
+        if (vco_run_start(sv0, j0, lo, hi, r0) & vco_run_start(sv1, j0, lo, hi, r1)) {
 #pragma unroll 1
-          for (int q = q0; q < q1; ++q) {
+          for (int q = 0; q < nq; ++q) {
             float ps[4], pq[4];
             vco_run_quad(sv0, r0, ps);
             vco_run_quad(sv1, r1, pq);
-            emit(f + 4 * q, ps, pq);
+            emit(rel_q + 4 * q, ps, pq);
           }
         } else {
-          // a chunk that meets a Nyquist-cap boundary evaluates each quad on its own
+          // a run that meets a Nyquist-cap boundary evaluates each quad on its own
 #pragma unroll 1
-          for (int q = q0; q < q1; ++q) {
+          for (int q = 0; q < nq; ++q) {
             float ps[4], pq[4];
-            vco_quad<false, true>(sv0, f + 4 * q - a, ps);
-            vco_quad<false, true>(sv1, f + 4 * q - a, pq);
+            vco_quad<false>(sv0, j0 + 4 * q, ps);
+            vco_quad<false>(sv1, j0 + 4 * q, pq);
 #pragma unroll
             for (int i = 0; i < 4; ++i) { ps[i] *= kTwoPiF; pq[i] *= kTwoPiF; }
-            emit(f + 4 * q, ps, pq);
+            emit(rel_q + 4 * q, ps, pq);
           }
         }
       }
@@ -854,7 +803,7 @@ __global__ void __launch_bounds__(NT, kCtasPerSm) render_fused_kernel(
         const int gq = min(G, (n_t - off0 + 3) >> 2);  // quads of the run inside the tile
         VcoRun r0, r1;
         // a run that meets a Nyquist-cap boundary evaluates each quad on its own
-        const bool run = vco_run_start(sv0, j0, 4 * G, r0) & vco_run_start(sv1, j0, 4 * G, r1);
+        const bool run = vco_run_start(sv0, j0, j0, j0 + 4 * G - 1, r0) & vco_run_start(sv1, j0, j0, j0 + 4 * G - 1, r1);
         if (kPeak) {
           // one loop for both cases (the peak variant's extra state leaves no
           // registers for two)
@@ -865,8 +814,8 @@ __global__ void __launch_bounds__(NT, kCtasPerSm) render_fused_kernel(
               vco_run_quad(sv0, r0, ps);
               vco_run_quad(sv1, r1, pq);
             } else {
-              vco_quad<false, true>(sv0, j0 + 4 * q, ps);
-              vco_quad<false, true>(sv1, j0 + 4 * q, pq);
+              vco_quad<false>(sv0, j0 + 4 * q, ps);
+              vco_quad<false>(sv1, j0 + 4 * q, pq);
 #pragma unroll
               for (int i = 0; i < 4; ++i) { ps[i] *= kTwoPiF; pq[i] *= kTwoPiF; }
             }
@@ -885,8 +834,8 @@ __global__ void __launch_bounds__(NT, kCtasPerSm) render_fused_kernel(
 #pragma unroll 1
           for (int q = 0; q < gq; ++q) {
             float ps[4], pq[4];
-            vco_quad<false, true>(sv0, j0 + 4 * q, ps);
-            vco_quad<false, true>(sv1, j0 + 4 * q, pq);
+            vco_quad<false>(sv0, j0 + 4 * q, ps);
+            vco_quad<false>(sv1, j0 + 4 * q, pq);
 #pragma unroll
             for (int i = 0; i < 4; ++i) { ps[i] *= kTwoPiF; pq[i] *= kTwoPiF; }
             emit(q, ps, pq);
