@@ -26,7 +26,11 @@
 //               already run in the other one.
 // Every mbarrier wait is bounded; on timeout the CTA records an error and
 // finishes.
+//
+// A product whose 128 x 64 tiles all fit the GPU at once and whose K is short
+// (the network's layers but the first) takes gemm_small instead: see there.
 
+#include <cooperative_groups.h>
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -472,6 +476,211 @@ __global__ void __launch_bounds__(256) splitk_reduce(const float* __restrict__ p
   }
 }
 
+// ---- products of one wave ----------------------------------------------------
+// C = A B^T for few 128 x 64 tiles and a short K, in one kernel: a cluster of
+// S CTAs takes a tile, each CTA a slice of K; the FP32 partial tiles stay in the
+// CTAs' shared memory and every CTA adds its share of the rows over the cluster,
+// in slice order, and applies the epilogue. What bounds such a product is the
+// chain launch - loads - MMAs - read-out, so it is spread over as many SMs as it
+// can use and each CTA's stages are all in flight at once. b_early: B is loaded
+// before the kernel ahead has finished (it does not write B).
+// 128 x 1024 x 1024 took 16 CTAs of 128 x 256 tiles and a reduction kernel.
+namespace cg = cooperative_groups;
+
+constexpr int SN = 64;            // tile columns
+constexpr int kSmallStages = 4;
+constexpr int kMaxSlices = 8;     // the portable cluster size
+constexpr int kPartLd = SN + 4;   // floats a row: rows 4 banks apart, 16-byte aligned
+
+struct __align__(1024) SmallSmem {
+  union {
+    __nv_bfloat16 a[kSmallStages][BM * BK];
+    float part[BM][kPartLd];                 // once the MMAs have read the operands
+  };
+  union {
+    __nv_bfloat16 b[kSmallStages][SN * BK];
+    __nv_bfloat16 t[SN][BM + 2];             // the finished rows, transposed
+  };
+  uint64_t full[kSmallStages];
+  uint64_t empty[kSmallStages];
+  uint64_t acc_full;
+  uint32_t tmem_base;
+  int failed;
+};
+// two CTAs on an SM, so that the next product of a chain starts beside this one
+static_assert(2 * (sizeof(SmallSmem) + 2048) <= 228 * 1024, "two CTAs per SM");
+
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+}
+
+__global__ void __launch_bounds__(kGemmThreads) gemm_small(
+    const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
+    GemmEpilogue epi, int M, int N, int nk, int slices, int kb_per, int b_early, unsigned int* err) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  SmallSmem& sm = *reinterpret_cast<SmallSmem*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int slice = (int)blockIdx.x % slices;  // = the CTA's rank in its cluster
+  const int tile = (int)blockIdx.x / slices;
+  const int tiles_n = (N + SN - 1) / SN;
+  const int m0 = (tile / tiles_n) * BM, n0 = (tile % tiles_n) * SN;
+  const int kb0 = slice * kb_per, kbs = min(nk - kb0, kb_per);  // >= 1
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kSmallStages; ++s) {
+      mbar_init(&sm.full[s], 1);
+      mbar_init(&sm.empty[s], 1);
+    }
+    mbar_init(&sm.acc_full, 1);
+    sm.failed = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(&sm.tmem_base)),
+                 "r"((uint32_t)SN));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = sm.tmem_base;
+
+  if (warp == 0 && lane == 0) {
+    const int early = b_early ? min(kbs, kSmallStages) : 0;  // the ring's first round: no stage to wait for
+    auto load_b = [&](int i) {
+      const int s = i % kSmallStages;
+      mbar_expect_tx(&sm.full[s], (uint32_t)((BM + SN) * BK * 2));
+      tma_load_2d(sm.b[s], &map_b, &sm.full[s], (kb0 + i) * BK, n0);
+    };
+    for (int i = 0; i < early; ++i) load_b(i);
+    pdl_wait();
+    pdl_release();
+    int issued = 0;
+    for (int i = 0; i < kbs; ++i) {
+      const int s = i % kSmallStages;
+      if (i >= early) {
+        if (!mbar_wait(&sm.empty[s], ((uint32_t)(i / kSmallStages) & 1u) ^ 1u)) { sm.failed = 1; break; }
+        load_b(i);
+      }
+      tma_load_2d(sm.a[s], &map_a, &sm.full[s], (kb0 + i) * BK, m0);
+      issued = i + 1;
+    }
+    // no copy of this CTA is in flight past this point
+    for (int i = max(0, issued - kSmallStages); i < issued; ++i)
+      if (!mbar_wait(&sm.full[i % kSmallStages], (uint32_t)(i / kSmallStages) & 1u)) sm.failed = 1;
+  } else {
+    pdl_wait();
+    pdl_release();
+  }
+  if (warp == 1 && lane == 0) {
+    constexpr uint32_t idesc = idesc_bf16_f32(BM, SN);
+    for (int i = 0; i < kbs; ++i) {
+      const int s = i % kSmallStages;
+      if (!mbar_wait(&sm.full[s], (uint32_t)(i / kSmallStages) & 1u)) { sm.failed = 1; break; }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t a0 = smem_u32(sm.a[s]), b0 = smem_u32(sm.b[s]);
+#pragma unroll
+      for (int kk = 0; kk < BK / 16; ++kk)
+        umma_bf16(tmem, smem_desc_sw128(a0 + kk * 32), smem_desc_sw128(b0 + kk * 32), idesc,
+                  (i != 0 || kk != 0) ? 1u : 0u);
+      umma_commit(&sm.empty[s]);
+    }
+    umma_commit(&sm.acc_full);
+  }
+  if (warp >= 2) {
+    // the accumulator to this CTA's part: warp = 32 rows, 32 columns; lane = row
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    if (!mbar_wait(&sm.acc_full, 0u)) sm.failed = 1;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    float v[32];
+    tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(32 * half), v);
+    float4* o = reinterpret_cast<float4*>(&sm.part[32 * q + lane][32 * half]);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) o[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  }
+  cluster_barrier();
+  if (warp >= 2) {
+    const int e0 = threadIdx.x - 64;
+    const int rows = min(BM, M - m0), per = (rows + slices - 1) / slices;
+    const int first = slice * per, count = max(0, min(per, rows - first));
+    const bool act = epi.kind != kEpiStoreF32;
+    const bool vec_f32 = (epi.ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(epi.out_f32) & 15) == 0;
+    const bool vec_b16 = (epi.ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(epi.out_bf16) & 7) == 0;
+    cg::cluster_group cluster = cg::this_cluster();
+    for (int e = e0; e < count * (SN / 4); e += 32 * kEpiWarps) {
+      const int rr = e / (SN / 4), r = first + rr, c = 4 * (e % (SN / 4));
+      float4 p[kMaxSlices];
+#pragma unroll
+      for (int s = 0; s < kMaxSlices; ++s)
+        if (s < slices)
+          p[s] = *reinterpret_cast<const float4*>(cluster.map_shared_rank(&sm.part[r][c], s));
+      float z[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int s = 0; s < kMaxSlices; ++s)
+        if (s < slices) { z[0] += p[s].x; z[1] += p[s].y; z[2] += p[s].z; z[3] += p[s].w; }
+      const int col = n0 + c;
+      const size_t at = (size_t)(m0 + r) * epi.ldc + col;
+      const bool whole = col + 3 < N;
+      __nv_bfloat16 b[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (epi.kind == kEpiReluGradBF16) {
+          z[i] = col + i < N && __bfloat162float(epi.gate[at + i]) > 0.f ? z[i] * epi.alpha : 0.f;
+        } else if (epi.kind == kEpiBiasActBF16) {
+          z[i] += epi.bias ? epi.bias[min(col + i, N - 1)] : 0.f;
+          if (epi.act == kActRelu) z[i] = fmaxf(z[i], 0.f);
+          else if (epi.act == kActSigmoid) z[i] = sigmoidf(z[i]);
+        } else {
+          z[i] *= epi.alpha;
+        }
+        b[i] = __float2bfloat16(z[i]);
+      }
+      if (epi.out_f32) {
+        if (whole && vec_f32) {
+          *reinterpret_cast<float4*>(epi.out_f32 + at) = make_float4(z[0], z[1], z[2], z[3]);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (col + i < N) epi.out_f32[at + i] = z[i];
+        }
+      }
+      if (act && epi.out_bf16) {
+        if (whole && vec_b16) {
+          *reinterpret_cast<uint2*>(epi.out_bf16 + at) = *reinterpret_cast<const uint2*>(b);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (col + i < N) epi.out_bf16[at + i] = b[i];
+        }
+      }
+      if (act && epi.out_bf16_t) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) sm.t[c + i][rr] = b[i];
+      }
+    }
+    if (act && epi.out_bf16_t) {
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
+      for (int e = e0; e < count * SN; e += 32 * kEpiWarps) {
+        const int c = e / count, rr = e - c * count;
+        if (n0 + c < N)
+          epi.out_bf16_t[(size_t)(n0 + c) * epi.ldc_t + m0 + first + rr] = sm.t[c][rr];
+      }
+    }
+  }
+  cluster_barrier();  // the parts have been read by every CTA
+  if (threadIdx.x == 0 && sm.failed) atomicOr(err, 1u);
+  if (warp == 1) {
+    __syncwarp();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                 "r"((uint32_t)SN));
+  }
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
                                   const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
                                   const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
@@ -510,7 +719,7 @@ bool make_map(CUtensorMap* map, const void* ptr, int rows, int cols, int ld, int
 // and whether each instantiation's dynamic shared-memory limit is raised.
 struct GemmDevice {
   int sms = 0;
-  bool attr128 = false, attr256 = false;
+  bool attr128 = false, attr256 = false, attr_small = false;
 };
 constexpr int kGemmMaxDevices = 64;
 std::mutex g_gemm_mutex;
@@ -541,6 +750,41 @@ cudaError_t gemm_device_setup(int* sms) {
   }
   *sms = d.sms;
   return cudaSuccess;
+}
+
+// The SM count of the current device, with gemm_small's shared memory set up.
+cudaError_t small_device_setup(int* sms) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= kGemmMaxDevices) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lock(g_gemm_mutex);
+  GemmDevice& d = g_gemm_dev[dev];
+  if (!d.attr_small) {
+    e = cudaFuncSetAttribute(gemm_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(sizeof(SmallSmem) + 1024));
+    if (e != cudaSuccess) return e;
+    d.attr_small = true;
+  }
+  if (d.sms == 0) {
+    e = cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+  }
+  *sms = d.sms;
+  return cudaSuccess;
+}
+
+// Slices of K for gemm_small (a power of two of CTAs a tile, at least two
+// k-blocks each, one CTA an SM at most, none empty), or 0 where the product is
+// not one for it.
+constexpr int kSmallMaxK = 64;  // k-blocks
+int small_slices(long long tiles, int nk, int sms, int* kb_per) {
+  if (tiles > sms || nk > kSmallMaxK) return 0;
+  int s = 1;
+  while (s < kMaxSlices && 2 * s * tiles <= sms && 4 * s <= nk) s *= 2;
+  *kb_per = (nk + s - 1) / s;
+  while ((s - 1) * *kb_per >= nk) s /= 2, *kb_per = (nk + s - 1) / s;
+  return s;
 }
 
 // K-slices for a product with `tiles` output tiles and nk k-blocks: enough
@@ -589,10 +833,25 @@ cudaError_t launch_bn(const CUtensorMap& ma, const CUtensorMap& mb, const GemmEp
 
 cudaError_t gemm_bf16(const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, int M,
                       int N, int K, const GemmEpilogue& epi, unsigned int* err, cudaStream_t st,
-                      float* splitk_ws, size_t splitk_bytes) {
+                      float* splitk_ws, size_t splitk_bytes, bool b_early) {
   if (M <= 0 || N <= 0 || K <= 0 || (K % 8) != 0) return cudaErrorInvalidValue;
-  const int bn = N > 128 ? 256 : 128;
   CUtensorMap ma, mb;
+  {
+    int sms = 0, kb_per = 0;
+    const cudaError_t e = small_device_setup(&sms);
+    if (e != cudaSuccess) return e;
+    const int nk = (K + BK - 1) / BK;
+    const long long tiles = (long long)((N + SN - 1) / SN) * ((M + BM - 1) / BM);
+    const int s = small_slices(tiles, nk, sms, &kb_per);
+    if (s > 0) {
+      if (!make_map(&ma, A, M, K, lda, BM) || !make_map(&mb, B, N, K, ldb, SN))
+        return cudaErrorInvalidValue;
+      return launch_pdl_cluster(gemm_small, dim3((unsigned)(tiles * s)), dim3(kGemmThreads),
+                                sizeof(SmallSmem) + 1024, st, (unsigned)s, ma, mb, epi, M, N, nk, s,
+                                kb_per, b_early ? 1 : 0, err);
+    }
+  }
+  const int bn = N > 128 ? 256 : 128;
   if (!make_map(&ma, A, M, K, lda, BM) || !make_map(&mb, B, N, K, ldb, bn))
     return cudaErrorInvalidValue;
   if (bn == 256) return launch_bn<256>(ma, mb, epi, M, N, K, splitk_ws, splitk_bytes, err, st);

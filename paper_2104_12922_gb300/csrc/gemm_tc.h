@@ -32,10 +32,13 @@ struct GemmEpilogue {
 // splitk_ws (splitk_bytes, device, 16-byte aligned) or NULL: when the output
 // has fewer 128 x BN tiles than the GPU has SMs, K is split into slices whose
 // FP32 partial products go there and a second kernel adds them in slice
-// order (deterministic) before the epilogue. NULL: no split.
+// order (deterministic) before the epilogue. NULL: no split, except inside a
+// cluster (gemm_small), which needs no workspace.
+// b_early: B is not written by the kernel just ahead on st, so that it may be
+// read before that kernel has finished.
 cudaError_t gemm_bf16(const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, int M,
                       int N, int K, const GemmEpilogue& epi, unsigned int* err, cudaStream_t st,
-                      float* splitk_ws = nullptr, size_t splitk_bytes = 0);
+                      float* splitk_ws = nullptr, size_t splitk_bytes = 0, bool b_early = false);
 
 // Workspace that lets gemm_bf16 split every product of at most max_m x max_n
 // outputs as far as it would (0 if the device cannot be queried).

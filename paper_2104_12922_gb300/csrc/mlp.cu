@@ -341,7 +341,7 @@ cudaError_t mlp_forward(const MlpLayout& L, char* base, const __nv_bfloat16* x, 
     }
     e = gemm_bf16(in, in_dim, reinterpret_cast<const __nv_bfloat16*>(base + L.wb[l]), in_dim, batch,
                   out, in_dim, ep, err, st, reinterpret_cast<float*>(base + L.splitk),
-                  L.splitk_bytes);
+                  L.splitk_bytes, l > 0);  // the kernel ahead of layer 0 may be its weights' Adam
     if (e != cudaSuccess) return e;
     in = reinterpret_cast<const __nv_bfloat16*>(base + L.h[l + 1 < 4 ? l + 1 : 3]);
     in_dim = out;
@@ -492,7 +492,7 @@ cudaError_t mlp_train_step(const MlpLayout& L, char* base, const MlpSide& side,
     eh.ldc_t = batch;
     if ((e = gemm_bf16(layer_grad(L, base, side, l).dz, ldz,
                        reinterpret_cast<const __nv_bfloat16*>(base + L.wt[l]), ldz, batch, in, ldz,
-                       eh, err, st, reinterpret_cast<float*>(base + L.splitk), L.splitk_bytes)) !=
+                       eh, err, st, reinterpret_cast<float*>(base + L.splitk), L.splitk_bytes, true)) !=
         cudaSuccess)
       return e;
   }
