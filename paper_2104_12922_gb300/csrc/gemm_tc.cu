@@ -401,79 +401,91 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tc(
   }
 }
 
-// Split-K reduction with the fused epilogue: C = sum over slices s = 0, 1, ...
-// of part[s] in that order, then the epilogue of `epi`. A block covers a
-// 16 x 32 output tile (32 x 8 threads, 2 rows each: 256 blocks for a
-// 128 x 1024 output); the transposed bf16 copy goes through shared memory
-// so both of its stores are coalesced.
-constexpr int kRedRows = 16;
-__global__ void __launch_bounds__(256) splitk_reduce(const float* __restrict__ part, int splits,
-                                                     int M, int N, GemmEpilogue epi) {
+// Split-K reduction with the fused epilogue. A block covers 8 x 32 outputs; each
+// of its 8 warps adds a contiguous eighth of the slices in order, all of its loads
+// in flight at once (five slices of two rows a thread for the 37 slices of 44160
+// inputs), and the eighths are added in order: the same sum in every run. It is
+// bound by the latency of those loads, which one warp for all slices paid five
+// times.
+constexpr int kRedRows = 8;
+constexpr int kRedWarps = 8;
+__global__ void __launch_bounds__(32 * kRedWarps) splitk_reduce(const float* __restrict__ part,
+                                                                int splits, int M, int N,
+                                                                GemmEpilogue epi) {
   pdl_wait();     // earlier kernels' writes are visible
   pdl_release();  // the next kernel may be scheduled
-  __shared__ float tile[kRedRows][33];
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const int c = blockIdx.x * 32 + tx, r0 = blockIdx.y * kRedRows;
+  __shared__ float4 sum[kRedWarps][kRedRows][8];
+  __shared__ __nv_bfloat16 tile[kRedRows][34];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int c0 = blockIdx.x * 32, r0 = blockIdx.y * kRedRows;
   const size_t slice = (size_t)M * N;
-  // the two rows' slices, eight at a time: 16 loads in flight per thread,
-  // added in slice order afterwards
-  const float* p[2];
-  bool ok[2];
+  {
+    constexpr int kPer = 5;  // slices in flight
+    const int per = (splits + kRedWarps - 1) / kRedWarps;
+    const int k0 = warp * per, k1 = min(splits, k0 + per);
+    const int c = c0 + 4 * (lane & 7), r = r0 + (lane >> 3);
+    const bool vec = (N & 3) == 0;
+    float4 acc[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+    for (int k = k0; k < k1; k += kPer) {
+      float4 t[2][kPer];
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int r = r0 + ty + 8 * i;
-    ok[i] = r < M && c < N;
-    p[i] = part + (size_t)(ok[i] ? r : 0) * N + (ok[i] ? c : 0);
-  }
-  float acc[2] = {0.f, 0.f};
-  int k = 0;
-  for (; k + 8 <= splits; k += 8) {
-    float t[2][8];
+      for (int u = 0; u < kPer; ++u)
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
-#pragma unroll
-      for (int i = 0; i < 2; ++i) t[i][u] = ok[i] ? p[i][(size_t)(k + u) * slice] : 0.f;
-#pragma unroll
-    for (int u = 0; u < 8; ++u)
-#pragma unroll
-      for (int i = 0; i < 2; ++i) acc[i] += t[i][u];
-  }
-  for (; k < splits; ++k)
-#pragma unroll
-    for (int i = 0; i < 2; ++i) acc[i] += ok[i] ? p[i][(size_t)k * slice] : 0.f;
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int r = r0 + ty + 8 * i;
-    float z = 0.f;
-    if (ok[i]) {
-      if (epi.kind == kEpiStoreF32) {
-        epi.out_f32[(size_t)r * epi.ldc + c] = acc[i] * epi.alpha;
-      } else {
-        if (epi.kind == kEpiReluGradBF16) {
-          z = __bfloat162float(epi.gate[(size_t)r * epi.ldc + c]) > 0.f ? acc[i] * epi.alpha : 0.f;
-        } else {
-          z = acc[i] + (epi.bias ? epi.bias[c] : 0.f);
-          if (epi.act == kActRelu) z = fmaxf(z, 0.f);
-          else if (epi.act == kActSigmoid) z = sigmoidf(z);
+        for (int i = 0; i < 2; ++i) {
+          const float* p = part + (size_t)(k + u) * slice + (size_t)(r + 4 * i) * N + c;
+          const bool ok = k + u < k1 && r + 4 * i < M;
+          t[i][u] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (vec) {
+            if (ok && c < N) t[i][u] = *reinterpret_cast<const float4*>(p);
+          } else if (ok) {
+            if (c < N) t[i][u].x = p[0];
+            if (c + 1 < N) t[i][u].y = p[1];
+            if (c + 2 < N) t[i][u].z = p[2];
+            if (c + 3 < N) t[i][u].w = p[3];
+          }
         }
-        const __nv_bfloat16 b = __float2bfloat16(z);
-        if (epi.out_bf16) epi.out_bf16[(size_t)r * epi.ldc + c] = b;
-        if (epi.out_f32) epi.out_f32[(size_t)r * epi.ldc + c] = z;
-        z = __bfloat162float(b);
-      }
+#pragma unroll
+      for (int u = 0; u < kPer; ++u)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          acc[i].x += t[i][u].x;
+          acc[i].y += t[i][u].y;
+          acc[i].z += t[i][u].z;
+          acc[i].w += t[i][u].w;
+        }
     }
-    tile[ty + 8 * i][tx] = z;
+    sum[warp][lane >> 3][lane & 7] = acc[0];
+    sum[warp][(lane >> 3) + 4][lane & 7] = acc[1];
+  }
+  __syncthreads();
+  // an output a thread: row = warp, column = lane
+  const int r = r0 + warp, c = c0 + lane;
+  const bool ok = r < M && c < N;
+  float a = 0.f, z = 0.f;
+#pragma unroll
+  for (int w = 0; w < kRedWarps; ++w) a += reinterpret_cast<const float*>(&sum[w][warp][0])[lane];
+  if (ok) {
+    if (epi.kind == kEpiStoreF32) {
+      epi.out_f32[(size_t)r * epi.ldc + c] = a * epi.alpha;
+    } else {
+      if (epi.kind == kEpiReluGradBF16) {
+        z = __bfloat162float(epi.gate[(size_t)r * epi.ldc + c]) > 0.f ? a * epi.alpha : 0.f;
+      } else {
+        z = a + (epi.bias ? epi.bias[c] : 0.f);
+        if (epi.act == kActRelu) z = fmaxf(z, 0.f);
+        else if (epi.act == kActSigmoid) z = sigmoidf(z);
+      }
+      if (epi.out_bf16) epi.out_bf16[(size_t)r * epi.ldc + c] = __float2bfloat16(z);
+      if (epi.out_f32) epi.out_f32[(size_t)r * epi.ldc + c] = z;
+    }
   }
   if (epi.kind == kEpiStoreF32 || !epi.out_bf16_t) return;
+  tile[warp][lane] = __float2bfloat16(z);
   __syncthreads();
-  // transposed: 16 rows of each of the 32 columns, lanes along the rows
-  const int rr = threadIdx.x & 15, cq = threadIdx.x >> 4;  // 16 rows x 16 column pairs
-#pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    const int cc = blockIdx.x * 32 + 2 * cq + j, r = r0 + rr;
-    if (cc < N && r < M)
-      epi.out_bf16_t[(size_t)cc * epi.ldc_t + r] = __float2bfloat16(tile[rr][2 * cq + j]);
-  }
+  // transposed: 8 rows of each of the 32 columns, lanes along the rows
+  const int rr = threadIdx.x & 7, cc = threadIdx.x >> 3;
+  if (c0 + cc < N && r0 + rr < M)
+    epi.out_bf16_t[(size_t)(c0 + cc) * epi.ldc_t + r0 + rr] = tile[rr][cc];
 }
 
 // ---- products of one wave ----------------------------------------------------

@@ -33,3 +33,30 @@ def test_small_product(m, n, k):
         assert ((c.double() - ref).abs() <= bar).all()
     assert torch.equal(outs[0], outs[1])
     syn.close()
+
+
+@pytest.mark.parametrize("m,n,k", [(5, 62, 8200), (129, 301, 4168), (9, 1024, 44160), (128, 258, 4104)])
+def test_split_product(m, n, k):
+    """Longer K: slices by CTA, added by the reduction kernel (rows of 8, columns of 32 or a ragged end of them)."""
+    import ctypes
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2104_12922_gb300 as pkg
+    syn = pkg.Synth(seconds=0.01, max_batch=1)
+    g = torch.Generator(device="cuda").manual_seed(m + 7 * n + k)
+    a = torch.randn(m, k, device="cuda", generator=g).to(torch.bfloat16)
+    b = torch.randn(n, k, device="cuda", generator=g).to(torch.bfloat16)
+    nb = ctypes.c_size_t()
+    assert pkg.lib().synth_gemm_bf16_workspace_size(syn.handle, m, n, ctypes.byref(nb)) == 0
+    ws = torch.empty(nb.value // 4 + 1, device="cuda")
+    c = torch.full((m, n + 1), float("nan"), device="cuda")
+    assert pkg.lib().synth_gemm_bf16_splitk(syn.handle, a.data_ptr(), k, b.data_ptr(), k, c.data_ptr(), n + 1, m, n, k,
+                                            1.0, ws.data_ptr(), nb.value,
+                                            torch.cuda.current_stream().cuda_stream) == 0
+    syn.sync()
+    assert torch.isnan(c[:, n]).all()
+    ref = a.double() @ b.double().T
+    bar = (a.double().abs() @ b.double().abs().T) * (k * 2.0 ** -22) + 1e-6
+    assert ((c[:, :n].double() - ref).abs() <= bar).all()
+    syn.close()
