@@ -13,6 +13,8 @@ def test_small_product(m, n, k):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     import paper_2104_12922_gb300 as pkg
+    from paper_2104_12922_gb300 import build as b_
+    b_.build()
     syn = pkg.Synth(seconds=0.01, max_batch=1)
     g = torch.Generator(device="cuda").manual_seed(m + 7 * n + k)
     a = torch.randn(m, k, device="cuda", generator=g).to(torch.bfloat16)
@@ -43,6 +45,8 @@ def test_split_product(m, n, k):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     import paper_2104_12922_gb300 as pkg
+    from paper_2104_12922_gb300 import build as b_
+    b_.build()
     syn = pkg.Synth(seconds=0.01, max_batch=1)
     g = torch.Generator(device="cuda").manual_seed(m + 7 * n + k)
     a = torch.randn(m, k, device="cuda", generator=g).to(torch.bfloat16)
