@@ -6,7 +6,7 @@
 // 4-operator FM architecture as in development (Sec. 3.2) and specifies no
 // more; parameter ranges and the stack are this library's choices.
 //
-// One CTA renders one voice's chunk of kFmChunk samples: it draws (or loads)
+// One CTA renders one voice's chunk of samples (fm_chunk): it draws (or loads)
 // the 30 normalized parameters, maps them, turns each operator's frequency
 // into a 64-bit fixed-point phase increment (the phase of sample n is the
 // exact product n x inc mod 2^64), evaluates the four envelopes at the
@@ -23,6 +23,7 @@
 // rounded to 2^-26 cycles where they were cut off at 2^-24).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "control_ff.cuh"
@@ -34,12 +35,13 @@ namespace synth {
 namespace {
 
 constexpr int kFmThreads = 256;
-constexpr int kFmChunk = 8192;                  // samples per CTA (a multiple of 4)
+constexpr int kFmCtasPerSm = 4;
 constexpr uint32_t kStreamFmParam = 2;
 
 struct FmConst {
   int64_t N, rate_a, rate_b;  // samples; R = rate_a / rate_b samples per control interval
   ff inv_cr;                  // 1 / control rate
+  int chunk;                  // samples per CTA (a multiple of 4)
   int max_pts;                // control points a chunk can span
   ff log2_440_over_sr;        // log2(440 / SR)
   alignas(16) FFTables T;     // float-float exp2 tables
@@ -154,7 +156,7 @@ __device__ __forceinline__ f32x2 sin2pi2(f32x2 t) {
                __uint_as_float(__float_as_uint(s1) ^ (__float_as_uint(m1) << 31)));
 }
 
-__global__ void __launch_bounds__(kFmThreads, 4) fm_render_kernel(const __grid_constant__ FmConst fc,
+__global__ void __launch_bounds__(kFmThreads, kFmCtasPerSm) fm_render_kernel(const __grid_constant__ FmConst fc,
                                                                uint64_t seed,
                                                                uint64_t batch_index, int batch,
                                                                const float* __restrict__ params_in,
@@ -171,9 +173,9 @@ __global__ void __launch_bounds__(kFmThreads, 4) fm_render_kernel(const __grid_c
   const int tid = threadIdx.x;
   const int v = blockIdx.y;
   const uint64_t g = batch_index * (uint64_t)batch + (uint64_t)v;
-  const int64_t s0 = (int64_t)blockIdx.x * kFmChunk;
+  const int64_t s0 = (int64_t)blockIdx.x * fc.chunk;
   const int64_t N = fc.N;
-  const int64_t s1 = min(s0 + (int64_t)kFmChunk, N);
+  const int64_t s1 = min(s0 + (int64_t)fc.chunk, N);
   // ---- parameters
   if (params_in == nullptr) {
     if (tid < 8) {
@@ -288,6 +290,40 @@ __global__ void __launch_bounds__(kFmThreads, 4) fm_render_kernel(const __grid_c
   }
 }
 
+// Samples per CTA of a launch: the cut of a voice that costs least, where a round
+// of resident CTAs first spends what kFmSetup samples cost on parameters and
+// envelopes (2.2 us), and a last round of fewer CTAs an SM takes the share of a
+// full one's time that kFmShare gives (the audio loop is bound by issue; fitted to
+// the times below); at equal cost the finer cut. 8192 samples for every launch
+// left the last round of CTAs part empty. 128 voices of 4 s: 71.8 -> 65.6 us (12600
+// samples; 9288: 69.7, 19600: 67.6, 4096: 79.5), 40: 28.6 -> 24.7, 16: 16.4 -> 13.0
+// (4644), one 10.3 -> 9.2; 128 of 1 s 26.3 -> 22.6, 100 of 2.3 s 38.0 -> 32.9. The
+// cuts meet the same samples: bit for bit as before.
+constexpr int kFmSetup = 1400;
+constexpr int kFmShare[kFmCtasPerSm] = {0, 40, 60, 82};  // percent
+constexpr int kFmDefaultChunk = 8192, kFmMaxChunk = 20480;
+constexpr int kFmMaxPoints = 1900;  // control points whose shared memory lets kFmCtasPerSm CTAs on an SM
+int fm_chunk(const VoiceConst& vc, int batch, int sms) {
+  const int64_t n = vc.n_samples;
+  const int64_t by_points = (int64_t)kFmMaxPoints * vc.rate_a / vc.rate_b;
+  if (by_points < kFmDefaultChunk) return kFmDefaultChunk;
+  const int64_t cap = std::min<int64_t>(kFmMaxChunk, by_points);
+  const int64_t first = (n + cap - 1) / cap;
+  int64_t best = 0, chunk = kFmDefaultChunk;
+  // CTAs a voice: 32 cuts at most, none below 1024 samples but the first (a launch
+  // of short voices takes as long as the call)
+  const int64_t last = std::max(first, std::min(first + 31, n / 1024));
+  for (int64_t c = first; c <= last; ++c) {
+    const int64_t len = (((n + c - 1) / c) + 3) / 4 * 4;
+    if (len > cap) continue;
+    const int64_t per_sm = ((n + len - 1) / len * batch + sms - 1) / sms;
+    const int64_t full = per_sm / kFmCtasPerSm, rest = per_sm % kFmCtasPerSm;
+    const int64_t cost = len * full + len * kFmShare[rest] / 100 + (full + (rest > 0)) * kFmSetup;
+    if (best == 0 || cost <= best) { best = cost; chunk = len; }
+  }
+  return (int)chunk;
+}
+
 }  // namespace
 
 cudaError_t launch_fm_render(const VoiceConst& vc, uint64_t seed, uint64_t batch_index, int batch,
@@ -295,6 +331,10 @@ cudaError_t launch_fm_render(const VoiceConst& vc, uint64_t seed, uint64_t batch
                              cudaStream_t stream) {
   if (batch <= 0) return cudaSuccess;
   if (batch > 65535) return cudaErrorInvalidValue;
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
   FmConst fc;
   fc.N = vc.n_samples;
   fc.rate_a = vc.rate_a;
@@ -302,16 +342,17 @@ cudaError_t launch_fm_render(const VoiceConst& vc, uint64_t seed, uint64_t batch
   fc.inv_cr = ff_from_double(1.0 / vc.control_rate);
   fc.log2_440_over_sr = vc.log2_440_over_sr;
   fc.T = vc.T;
-  fc.max_pts = (int)((int64_t)kFmChunk * vc.rate_b / vc.rate_a) + 3;
+  fc.chunk = fm_chunk(vc, batch, sms);
+  fc.max_pts = (int)((int64_t)fc.chunk * vc.rate_b / vc.rate_a) + 3;
   const size_t smem = sizeof(float) * 6 * (size_t)fc.max_pts;
   if (smem > 200 * 1024) return cudaErrorInvalidValue;
   if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(fm_render_kernel,
+    e = cudaFuncSetAttribute(fm_render_kernel,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)smem);
+                             (int)smem);
     if (e != cudaSuccess) return e;
   }
-  const dim3 grid((unsigned)((vc.n_samples + kFmChunk - 1) / kFmChunk), (unsigned)batch);
+  const dim3 grid((unsigned)((vc.n_samples + fc.chunk - 1) / fc.chunk), (unsigned)batch);
   fm_render_kernel<<<grid, kFmThreads, smem, stream>>>(fc, seed, batch_index, batch, params_in,
                                                        audio, params_out);
   return cudaGetLastError();
