@@ -442,14 +442,14 @@ struct OlaRes {
   const float* part;  // [batch][groups][seg]
   int n, hop, G, groups, seg, F;
 };
+constexpr int kMrRes = 3;  // resolutions
 struct OlaArgs {
-  OlaRes r[8];
-  int n_res;
+  OlaRes r[kMrRes];
 };
 
 __device__ __forceinline__ float ola_sample(const OlaArgs& a, int N, int v, int s) {
   float acc = 0.f;
-  for (int k = 0; k < a.n_res; ++k) {
+  for (int k = 0; k < kMrRes; ++k) {
     const OlaRes& R = a.r[k];
     const int pad = R.n / 2, stride = R.G * R.hop;
     const float* pv = R.part + (size_t)v * R.groups * R.seg;
@@ -472,34 +472,68 @@ __device__ __forceinline__ float ola_sample(const OlaArgs& a, int N, int v, int 
   return acc;
 }
 
+// A voice's loss: the sum of its items, by one warp. The lanes load 32 items at a
+// time, whose sum is taken in item order (one thread that loaded them one by one
+// took 5.6 us for the 33 items of 1 s).
+struct MrLossItems {
+  const double* item[kMrRes];
+  int groups[kMrRes];
+};
+__device__ __forceinline__ void voice_loss(const MrLossItems& li, int v, double* loss_voice) {
+  const int lane = threadIdx.x & 31;
+  double s = 0.0;
+  for (int r = 0; r < kMrRes; ++r)
+    for (int g = 0; g < li.groups[r]; g += 32) {
+      const int m = min(32, li.groups[r] - g);
+      const double x = lane < m ? li.item[r][(size_t)v * li.groups[r] + g + lane] : 0.0;
+      for (int j = 0; j < m; ++j) s += __shfl_sync(0xffffffffu, x, j);
+    }
+  if (lane == 0) loss_voice[v] = s;
+}
+
 // Four samples per thread: away from the ends (no reflected positions) the
 // four padded positions s + n/2 share their items and segment bounds (all
 // multiples of 4), so each covering segment contributes one 16-byte load.
-__global__ void mr_ola_gather(OlaArgs a, int N, int pad_max, float* __restrict__ grad) {
+// Segments start every kMrStride positions at every resolution; position p lies
+// in that of item i = p / kMrStride (the last at most) and, for 3/4 n positions,
+// in the one before. The kernel was bound by its index arithmetic (475
+// instructions for at most six loads); all loads are in flight at once. One block
+// of each voice's adds up its loss, which was a kernel of its own.
+constexpr int kMrStride = 16 * 32 * kWarpsMr;  // G hop = (32 kWarpsMr / R) (16 R)
+__global__ void mr_ola_gather(const __grid_constant__ OlaArgs a, const __grid_constant__ MrLossItems li,
+                              int N, int pad_max, float* __restrict__ grad,
+                              double* __restrict__ loss_voice) {
   const int v = blockIdx.y;
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x < 32) voice_loss(li, v, loss_voice);
   const int n4 = (N + 3) / 4;
   const bool vec = (N & 3) == 0 && (reinterpret_cast<uintptr_t>(grad) & 15) == 0;
   for (int i4 = blockIdx.x * blockDim.x + threadIdx.x; i4 < n4; i4 += gridDim.x * blockDim.x) {
     const int s0 = 4 * i4;
     if (vec && s0 > pad_max && s0 + 3 <= N - 2 - pad_max) {
       float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int k = 0; k < a.n_res; ++k) {
+      float4 t[kMrRes][2];
+#pragma unroll
+      for (int k = 0; k < kMrRes; ++k) {
         const OlaRes& R = a.r[k];
-        const int stride = R.G * R.hop, p0 = s0 + R.n / 2;
-        const float* pv = R.part + (size_t)v * R.groups * R.seg;
-        const int i = min(p0 / stride, R.groups - 1);
-        for (int q = i; q >= 0 && q >= i - 1; --q) {
-          const int off = p0 - q * stride;
-          const int len = (min(R.G, R.F - q * R.G) - 1) * R.hop + R.n;
-          if (off >= 0 && off < len) {
-            const float4 t = *reinterpret_cast<const float4*>(pv + (size_t)q * R.seg + off);
-            acc.x += t.x;
-            acc.y += t.y;
-            acc.z += t.z;
-            acc.w += t.w;
-          }
-        }
+        const int p0 = s0 + R.n / 2;
+        const int i = min(p0 / kMrStride, R.groups - 1);
+        const int off = p0 - i * kMrStride;
+        const float* ps = R.part + ((size_t)v * R.groups + i) * R.seg + off;
+        t[k][0] = t[k][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (off < (min(R.G, R.F - i * R.G) - 1) * R.hop + R.n) t[k][0] = *reinterpret_cast<const float4*>(ps);
+        // item i - 1 has all of its frames
+        if (i >= 1 && off + kMrStride < kMrStride - R.hop + R.n)
+          t[k][1] = *reinterpret_cast<const float4*>(ps - R.seg + kMrStride);
       }
+#pragma unroll
+      for (int k = 0; k < kMrRes; ++k)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          acc.x += t[k][u].x;
+          acc.y += t[k][u].y;
+          acc.z += t[k][u].z;
+          acc.w += t[k][u].w;
+        }
       *reinterpret_cast<float4*>(grad + (size_t)v * N + s0) = acc;
     } else {
       for (int s = s0; s < min(s0 + 4, N); ++s) grad[(size_t)v * N + s] = ola_sample(a, N, v, s);
@@ -642,19 +676,9 @@ struct MrLayout {
 // Per-voice loss: the work items' partial sums added in a fixed order
 // (resolution, then frame group), so the total does not depend on which
 // CTA finished first.
-struct MrLossItems {
-  const double* item[8];
-  int groups[8];
-  int n_res;
-};
-
 __global__ void mr_loss_reduce(MrLossItems li, int batch, double* __restrict__ loss_voice) {
-  const int v = blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= batch) return;
-  double s = 0.0;
-  for (int r = 0; r < li.n_res; ++r)
-    for (int g = 0; g < li.groups[r]; ++g) s += li.item[r][(size_t)v * li.groups[r] + g];
-  loss_voice[v] = s;
+  const int v = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+  if (v < batch) voice_loss(li, v, loss_voice);
 }
 
 MrLayout mr_layout(int64_t N, int batch, const int* n_ffts, int n_res, void* ws) {
@@ -689,7 +713,7 @@ cudaError_t mrstft_loss_grad(const float* x, const float* y, int64_t N, int batc
                              const int* n_ffts, int n_res, float eps, bool target_ready,
                              double* loss_voice_out, float* grad_x, void* ws, unsigned int* err,
                              cudaStream_t st) {
-  if (n_res < 1 || n_res > 8) return cudaErrorInvalidValue;
+  if (n_res != kMrRes) return cudaErrorInvalidValue;
   for (int r = 0; r < n_res; ++r)  // reflect padding needs more samples than half a frame
     if (r_of(n_ffts[r]) == 0 || N <= n_ffts[r] / 2 || N >= (int64_t)1 << 31)
       return cudaErrorInvalidValue;
@@ -707,8 +731,6 @@ cudaError_t mrstft_loss_grad(const float* x, const float* y, int64_t N, int batc
   }
   OlaArgs ola;
   MrLossItems li;
-  li.n_res = n_res;
-  ola.n_res = n_res;
   for (int r = 0; r < n_res; ++r) {
     const int n = n_ffts[r], F = stft_frames(N, n);
     const float scale = 1.0f / (float)((int64_t)F * (n / 2 + 1));
@@ -721,14 +743,15 @@ cudaError_t mrstft_loss_grad(const float* x, const float* y, int64_t N, int batc
     ola.r[r] = OlaRes{L.part[r], n, n / 4, mr_group(n), (F + mr_group(n) - 1) / mr_group(n),
                       mr_seg(n), F};
   }
+  double* loss_voice = loss_voice_out ? loss_voice_out : L.loss_voice;
   if (grad_x) {
     int pad_max = 0;
     for (int r = 0; r < n_res; ++r) pad_max = std::max(pad_max, n_ffts[r] / 2);
     dim3 go((unsigned)std::min<int64_t>((N / 4 + 255) / 256 + 1, 1024), (unsigned)batch);
-    mr_ola_gather<<<go, 256, 0, st>>>(ola, (int)N, pad_max, grad_x);
+    mr_ola_gather<<<go, 256, 0, st>>>(ola, li, (int)N, pad_max, grad_x, loss_voice);
+  } else {
+    mr_loss_reduce<<<(batch + 3) / 4, 128, 0, st>>>(li, batch, loss_voice);
   }
-  mr_loss_reduce<<<(batch + 127) / 128, 128, 0, st>>>(li, batch,
-                                                     loss_voice_out ? loss_voice_out : L.loss_voice);
   return cudaGetLastError();
 }
 
