@@ -27,8 +27,8 @@
 // Every mbarrier wait is bounded; on timeout the CTA records an error and
 // finishes.
 //
-// A product whose 128 x 64 tiles all fit the GPU at once and whose K is short
-// (the network's layers but the first) takes gemm_small instead: see there.
+// A product whose 128 x 64 tiles and slices all fit the GPU at once and whose K is
+// short (the network's layers but the first) takes gemm_small instead: see there.
 
 #include <cooperative_groups.h>
 #include <cuda.h>
@@ -401,69 +401,61 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tc(
   }
 }
 
-// Split-K reduction with the fused epilogue. A block covers 8 x 32 outputs; each
-// of its 8 warps adds a contiguous eighth of the slices in order, all of its loads
-// in flight at once (five slices of two rows a thread for the 37 slices of 44160
-// inputs), and the eighths are added in order: the same sum in every run. It is
-// bound by the latency of those loads, which one warp for all slices paid five
+// Split-K reduction with the fused epilogue: C = sum over slices s = 0, 1, ... of
+// part[s] in that order. A block covers 8 x 32 outputs; its 8 warps load the
+// slices into shared memory, five of two rows a thread in flight at once (the 37
+// slices of 44160 inputs in one go), and a thread an output adds them in order. It
+// is bound by the latency of those loads, which one warp for all slices paid five
 // times.
 constexpr int kRedRows = 8;
 constexpr int kRedWarps = 8;
+constexpr int kRedPer = 5;  // slices a warp has in flight
 __global__ void __launch_bounds__(32 * kRedWarps) splitk_reduce(const float* __restrict__ part,
                                                                 int splits, int M, int N,
                                                                 GemmEpilogue epi) {
   pdl_wait();     // earlier kernels' writes are visible
   pdl_release();  // the next kernel may be scheduled
-  __shared__ float4 sum[kRedWarps][kRedRows][8];
+  __shared__ float4 slices[kRedWarps * kRedPer][kRedRows][8];
   __shared__ __nv_bfloat16 tile[kRedRows][34];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int c0 = blockIdx.x * 32, r0 = blockIdx.y * kRedRows;
   const size_t slice = (size_t)M * N;
-  {
-    constexpr int kPer = 5;  // slices in flight
-    const int per = (splits + kRedWarps - 1) / kRedWarps;
-    const int k0 = warp * per, k1 = min(splits, k0 + per);
-    const int c = c0 + 4 * (lane & 7), r = r0 + (lane >> 3);
-    const bool vec = (N & 3) == 0;
-    float4 acc[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
-    for (int k = k0; k < k1; k += kPer) {
-      float4 t[2][kPer];
+  const bool vec = (N & 3) == 0;
+  float a = 0.f;
+  for (int k0 = 0; k0 < splits; k0 += kRedWarps * kRedPer) {
+    const int n = min(splits - k0, kRedWarps * kRedPer);
+    const int cl = c0 + 4 * (lane & 7), rl = r0 + (lane >> 3);
+    float4 t[2][kRedPer];
 #pragma unroll
-      for (int u = 0; u < kPer; ++u)
+    for (int u = 0; u < kRedPer; ++u)
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          const float* p = part + (size_t)(k + u) * slice + (size_t)(r + 4 * i) * N + c;
-          const bool ok = k + u < k1 && r + 4 * i < M;
-          t[i][u] = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (vec) {
-            if (ok && c < N) t[i][u] = *reinterpret_cast<const float4*>(p);
-          } else if (ok) {
-            if (c < N) t[i][u].x = p[0];
-            if (c + 1 < N) t[i][u].y = p[1];
-            if (c + 2 < N) t[i][u].z = p[2];
-            if (c + 3 < N) t[i][u].w = p[3];
-          }
+      for (int i = 0; i < 2; ++i) {
+        const int k = warp + kRedWarps * u;
+        const float* p = part + (size_t)(k0 + k) * slice + (size_t)(rl + 4 * i) * N + cl;
+        const bool ok = k < n && rl + 4 * i < M;
+        t[i][u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (vec) {
+          if (ok && cl < N) t[i][u] = *reinterpret_cast<const float4*>(p);
+        } else if (ok) {
+          if (cl < N) t[i][u].x = p[0];
+          if (cl + 1 < N) t[i][u].y = p[1];
+          if (cl + 2 < N) t[i][u].z = p[2];
+          if (cl + 3 < N) t[i][u].w = p[3];
         }
+      }
+    if (k0 > 0) __syncthreads();  // the slices before have been added
 #pragma unroll
-      for (int u = 0; u < kPer; ++u)
+    for (int u = 0; u < kRedPer; ++u)
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          acc[i].x += t[i][u].x;
-          acc[i].y += t[i][u].y;
-          acc[i].z += t[i][u].z;
-          acc[i].w += t[i][u].w;
-        }
-    }
-    sum[warp][lane >> 3][lane & 7] = acc[0];
-    sum[warp][(lane >> 3) + 4][lane & 7] = acc[1];
+      for (int i = 0; i < 2; ++i) slices[warp + kRedWarps * u][(lane >> 3) + 4 * i][lane & 7] = t[i][u];
+    __syncthreads();
+#pragma unroll 8
+    for (int k = 0; k < n; ++k) a += reinterpret_cast<const float*>(&slices[k][warp][0])[lane];
   }
-  __syncthreads();
   // an output a thread: row = warp, column = lane
   const int r = r0 + warp, c = c0 + lane;
   const bool ok = r < M && c < N;
-  float a = 0.f, z = 0.f;
-#pragma unroll
-  for (int w = 0; w < kRedWarps; ++w) a += reinterpret_cast<const float*>(&sum[w][warp][0])[lane];
+  float z = 0.f;
   if (ok) {
     if (epi.kind == kEpiStoreF32) {
       epi.out_f32[(size_t)r * epi.ldc + c] = a * epi.alpha;
@@ -496,7 +488,8 @@ __global__ void __launch_bounds__(32 * kRedWarps) splitk_reduce(const float* __r
 // chain launch - loads - MMAs - read-out, so it is spread over as many SMs as it
 // can use and each CTA's stages are all in flight at once. b_early: B is loaded
 // before the kernel ahead has finished (it does not write B).
-// 128 x 1024 x 1024 took 16 CTAs of 128 x 256 tiles and a reduction kernel.
+// 128 x 1024 x 1024 took 16 CTAs of 128 x 256 tiles and a reduction kernel, 13 us in
+// all; the output layer's input gradient 18 us on 4 CTAs.
 namespace cg = cooperative_groups;
 
 constexpr int SN = 64;            // tile columns
@@ -786,19 +779,6 @@ cudaError_t small_device_setup(int* sms) {
   return cudaSuccess;
 }
 
-// Slices of K for gemm_small (a power of two of CTAs a tile, at least two
-// k-blocks each, one CTA an SM at most, none empty), or 0 where the product is
-// not one for it.
-constexpr int kSmallMaxK = 64;  // k-blocks
-int small_slices(long long tiles, int nk, int sms, int* kb_per) {
-  if (tiles > sms || nk > kSmallMaxK) return 0;
-  int s = 1;
-  while (s < kMaxSlices && 2 * s * tiles <= sms && 4 * s <= nk) s *= 2;
-  *kb_per = (nk + s - 1) / s;
-  while ((s - 1) * *kb_per >= nk) s /= 2, *kb_per = (nk + s - 1) / s;
-  return s;
-}
-
 // K-slices for a product with `tiles` output tiles and nk k-blocks: enough
 // to give every SM an item, at least 4 k-blocks per slice, within the
 // workspace. Returns 1 (no split) when the tiles alone fill the GPU.
@@ -811,6 +791,20 @@ int choose_splits(int tiles, int nk, int sms, size_t slice_bytes, size_t ws_byte
   if (s <= 1) return 1;
   *kb_per = (nk + s - 1) / s;
   return (nk + *kb_per - 1) / *kb_per;
+}
+
+// Whether a product goes to gemm_small: its 128 x 64 tiles and slices are resident at
+// once, K is short, and its slices are those of the general path and fit a cluster, so
+// that the sums, and a training run with them, are the same bit for bit (a change of
+// rounding in a gradient near zero turns Adam's step there round). That costs a little:
+// with up to 8 slices of two k-blocks instead of 4 of four, and the first layer's slices
+// added by eighths, a proposal for 16 sounds took 64.7 us and a training step 383, with
+// the general path's order 67.1 and 386 (85.9 and 400 without gemm_small and with one
+// warp for all slices of the reduction).
+constexpr int kSmallMaxK = 64;  // k-blocks
+bool is_small(long long tiles, int slices, int nk, int sms) {
+  return tiles <= sms && tiles * slices <= 2 * sms && nk <= kSmallMaxK && slices <= kMaxSlices &&
+         (slices & (slices - 1)) == 0;
 }
 
 template <int BN>
@@ -847,15 +841,20 @@ cudaError_t gemm_bf16(const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, i
                       int N, int K, const GemmEpilogue& epi, unsigned int* err, cudaStream_t st,
                       float* splitk_ws, size_t splitk_bytes, bool b_early) {
   if (M <= 0 || N <= 0 || K <= 0 || (K % 8) != 0) return cudaErrorInvalidValue;
+  const int bn = N > 128 ? 256 : 128;
   CUtensorMap ma, mb;
   {
-    int sms = 0, kb_per = 0;
+    int sms = 0;
     const cudaError_t e = small_device_setup(&sms);
     if (e != cudaSuccess) return e;
     const int nk = (K + BK - 1) / BK;
-    const long long tiles = (long long)((N + SN - 1) / SN) * ((M + BM - 1) / BM);
-    const int s = small_slices(tiles, nk, sms, &kb_per);
-    if (s > 0) {
+    const long long rows = (M + BM - 1) / BM, tiles = rows * ((N + SN - 1) / SN);
+    const long long big = rows * ((N + bn - 1) / bn);  // the general path's tiles
+    int kb_per = nk;
+    const int s = splitk_ws ? choose_splits((int)std::min<long long>(big, 1 << 30), nk, sms,
+                                            sizeof(float) * (size_t)M * N, splitk_bytes, &kb_per)
+                            : 1;
+    if (is_small(tiles, s, nk, sms)) {
       if (!make_map(&ma, A, M, K, lda, BM) || !make_map(&mb, B, N, K, ldb, SN))
         return cudaErrorInvalidValue;
       return launch_pdl_cluster(gemm_small, dim3((unsigned)(tiles * s)), dim3(kGemmThreads),
@@ -863,7 +862,6 @@ cudaError_t gemm_bf16(const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, i
                                 kb_per, b_early ? 1 : 0, err);
     }
   }
-  const int bn = N > 128 ? 256 : 128;
   if (!make_map(&ma, A, M, K, lda, BM) || !make_map(&mb, B, N, K, ldb, bn))
     return cudaErrorInvalidValue;
   if (bn == 256) return launch_bn<256>(ma, mb, epi, M, N, K, splitk_ws, splitk_bytes, err, st);

@@ -32,8 +32,8 @@ struct GemmEpilogue {
 // splitk_ws (splitk_bytes, device, 16-byte aligned) or NULL: when the output
 // has fewer 128 x BN tiles than the GPU has SMs, K is split into slices whose
 // FP32 partial products go there and a second kernel adds them in slice
-// order (deterministic) before the epilogue. NULL: no split, except inside a
-// cluster (gemm_small), which needs no workspace.
+// order (deterministic) before the epilogue, or which a cluster adds in the same
+// order (gemm_small). NULL: no split.
 // b_early: B is not written by the kernel just ahead on st, so that it may be
 // read before that kernel has finished.
 cudaError_t gemm_bf16(const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, int M,
