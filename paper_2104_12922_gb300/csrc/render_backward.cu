@@ -29,7 +29,15 @@
 // integers (an FP64 scan waits on the narrow FP64 pipe), and an interval's 21
 // sums are added up over 8 lanes, not 32. Kernels of the plain form's modules,
 // a warp per interval and a scan kernel that handed FP64 point adjoints on took
-// 110.6 us; now 77.3 us (the three under a profiler: 20, 33 and 30).
+// 110.6 us; now 78.0 us.
+//
+// Precision: every value that goes from one kernel to the next is rounded to float
+// once, from float-float (parameters, envelopes, mixer gains and outputs, phases)
+// or FP64 (a point's pitch adjoint, whose two ends and running sums cancel).
+// Mixer outputs as FP32 sums and pitch adjoints rounded before they were added
+// took 76.6 us, and their error against 64 bits was up to 1.7 times that of the
+// modules' kernels over a batch (10 times for a voice); now it is theirs, 7.6e-6
+// over 1280 voices of 0.1 s and 8.2e-6 over 872 of 0.1 to 2 s.
 
 #include "control_ff.cuh"
 #include "internal.h"
@@ -156,11 +164,13 @@ __global__ void __launch_bounds__(kCT) bwd_recompute(const __grid_constant__ Voi
   if (tid < 16) {
     voice_ff_fill(s.V, s.y, tid);
   } else if (tid == 32) {
-    const float l0 = ff_to_float(s.y[kMix]), l1 = ff_to_float(s.y[kMix + 1]),
-                l2 = ff_to_float(s.y[kMix + 2]);
-    const float inv = 1.f / fmaxf(1.f, l0 + l1 + l2);
+    const ff sum = ff_add(ff_add(s.y[kMix], s.y[kMix + 1]), s.y[kMix + 2]);
+    const ff inv = ff_lt(sum, ff_make(1.f)) ? ff_make(1.f) : ff_rcp(sum);
+    float g[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) g[c] = ff_to_float(ff_mul(s.y[kMix + c], inv));
     *reinterpret_cast<float4*>(b.mix + (size_t)v * 4) =
-        make_float4(l0 * inv, l1 * inv, l2 * inv, ff_to_float(s.y[kSqr + 3]));
+        make_float4(g[0], g[1], g[2], ff_to_float(s.y[kSqr + 3]));
   } else if (tid >= 64 && tid < 68) {
     const int slot[4] = {kLfo + 2, kLfo + 8 + 2, kSine + 2, kSqr + 2};
     s.p0[tid - 64] = ff_to_fix64(ff_mul(s.y[slot[tid - 64]], vc.inv_2pi));
@@ -196,24 +206,17 @@ __global__ void __launch_bounds__(kCT) bwd_recompute(const __grid_constant__ Voi
     __syncthreads();
     if (p <= nseg) {
       const ff src[4] = {s.env[0][p], s.env[1][p], s.env[3][p], s.env[5][p]};
-      ff m = V.pitch_base[half];
+      // the mixer's outputs, two or three a half (the pitch one, then amplitudes): sums
+      // in float-float, rounded once
+#pragma unroll 1
+      for (int j = 2 * half; j < 2 + 3 * half; ++j) {
+        ff acc = ff_mul(V.mod_w[0][j], src[0]);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) m = ff_add(m, ff_mul(V.pitch_w[half][q], src[q]));
-      s.env[2 + 2 * half][p] = m;
-      // the mixer's outputs as floats, two or three a half: the pitch one, then amplitudes
-      auto put = [&](int j, const float w[4]) {
-        float acc = w[0] * ff_to_float(src[0]);
-#pragma unroll
-        for (int q = 1; q < 4; ++q) acc = fmaf(w[q], ff_to_float(src[q]), acc);
-        b.dest[((size_t)v * 5 + j) * P + base + p] = acc;
-      };
-      const int jp = 2 * half;
-      float wp[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) wp[q] = ff_to_float(V.mod_w[q][jp]) * ff_to_float(V.inv_norm[jp]);
-      put(jp, wp);
-      put(jp + 1, V.amp_w[half]);
-      if (half == 1) put(4, V.amp_w[2]);
+        for (int q = 1; q < 4; ++q) acc = ff_add(acc, ff_mul(V.mod_w[q][j], src[q]));
+        acc = ff_mul(acc, V.inv_norm[j]);
+        b.dest[((size_t)v * 5 + j) * P + base + p] = ff_to_float(acc);
+        if (j == 2 * half) s.env[j + 2][p] = ff_add(V.pitch_base[half], ff_mul(V.depth[half], acc));
+      }
     }
     __syncthreads();
     ff adv = ff_make(0.f);
@@ -236,7 +239,9 @@ __global__ void __launch_bounds__(kCT) bwd_recompute(const __grid_constant__ Voi
         vco_carry + half_scan(s, p < nseg ? ff_to_fix64(adv) : 0ull, tot);
     vco_carry += tot;
     if (p < nseg && in_bounds(hdr, base + p, K)) {
-      sv.phase0 = fix64_to_float(start);
+      // from 48 bits: a phase cut to 32 bits first rounds the other way in 1% of the intervals,
+      // which a steep square-saw shows
+      sv.phase0 = ff_to_float(fix64_to_ff(start));
       b.seg[((size_t)v * 2 + half) * K + base + p] = sv;
     }
     __syncthreads();  // the chunk's envelopes are done with
@@ -264,12 +269,12 @@ __device__ __forceinline__ void vco_quad_and_inc(const SegVco& s, int j0, float 
     const float c = in_b ? s.cB : s.cA;
     const bool lin = (s.jc_flags >> (in_b ? 17 : 16)) & 1;
     const bool cap = (s.jc_flags >> (in_b ? 19 : 18)) & 1;
-    const float z = (float)(j0 - (in_b ? jc : 0)) * (lin ? 0.f : s.x);
-    const float r = lin ? 1.f : s.q2 - 1.f;
-    inc[0] = cap ? 0.f : fmaf(c, expm1_phase(z), c);
-    inc[1] = inc[0] * r;
-    inc[2] = inc[1] * r;
-    inc[3] = inc[2] * r;
+    const float x = lin ? 0.f : s.x;
+    const float e1 = expm1_phase(x);  // q2 - 2 has lost its last bits
+    inc[0] = cap ? 0.f : fmaf(c, expm1_phase((float)(j0 - (in_b ? jc : 0)) * x), c);
+    inc[1] = fmaf(inc[0], e1, inc[0]);
+    inc[2] = fmaf(inc[1], e1, inc[1]);
+    inc[3] = fmaf(inc[2], e1, inc[2]);
   } else {
     bool cap[4];
     vco_inc_quad(s, j0, inc, cap);
@@ -339,7 +344,7 @@ __global__ void __launch_bounds__(kST, 6) bwd_samples(const __grid_constant__ Vo
     for (int t = 3; t >= 0; --t) {
       const bool on = j0 + t < Rk;
       const float go = go4[t];
-      const float fj = (float)(j0 + t) * invR;
+      const float fj = (float)(j0 + t) * invR, fl = 1.f - fj;
       float A[3];
 #pragma unroll
       for (int c = 0; c < 3; ++c) A[c] = fmaf(fj, da[c], a0[c]);
@@ -354,7 +359,7 @@ __global__ void __launch_bounds__(kST, 6) bwd_samples(const __grid_constant__ Vo
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         const float dA = gg[c] * x[c];
-        acc[10 + c] = fmaf(dA, 1.f - fj, acc[10 + c]);
+        acc[10 + c] = fmaf(dA, fl, acc[10 + c]);
         acc[13 + c] = fmaf(dA, fj, acc[13 + c]);
         acc[17 + c] = fmaf(go * A[c], x[c], acc[17 + c]);
       }
@@ -367,7 +372,7 @@ __global__ void __launch_bounds__(kST, 6) bwd_samples(const __grid_constant__ Vo
       acc[20] = fmaf(gA1 * ip * th * itk, cs - 1.f, acc[20]);
 #pragma unroll
       for (int o = 0; o < 2; ++o) {
-        const float w = on ? inc[o][t] : 0.f, wr = w * fj, wl = w - wr;
+        const float w = on ? inc[o][t] : 0.f, wr = w * fj, wl = w * fl;
         acc[5 * o + 1] = fmaf(wl, ls[o], acc[5 * o + 1]);
         acc[5 * o + 2] += wl;
         acc[5 * o + 3] = fmaf(wr, ls[o], acc[5 * o + 3]);
@@ -550,7 +555,7 @@ __global__ void __launch_bounds__(kBC) bwd_control(const __grid_constant__ Voice
   if (!in_bounds(hdr, v, batch)) return;
   const float inv_cr = (float)(1.0 / vc.control_rate);
   const float inv_2pi = 0.15915494309189533577f;
-  const float l12 = (float)(kLn2 / 12.0);
+  const double l12 = kLn2 / 12.0;
   float* gyw = gyw_all[threadIdx.x >> 5];
   for (int i = threadIdx.x; i < kGY * (kBC / 32); i += kBC) (&gyw_all[0][0])[i] = 0.f;
   for (int i = threadIdx.x; i < kNumParams; i += kBC) yv[i] = buf.y[(size_t)v * 80 + i];
@@ -614,28 +619,31 @@ __global__ void __launch_bounds__(kBC) bwd_control(const __grid_constant__ Voice
     }
     const float src[4] = {e[0], e[1], lfo[0], lfo[1]};
     // the point's pitch and amplitude adjoints: the left end of interval k and the
-    // right end of interval k - 1
+    // right end of interval k - 1, the pitch ones' sums in FP64 (they cancel)
     float gk[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+    double gm0 = 0.0, gm1 = 0.0;
     if (ok && k < K) {
       const float* st = stat + (size_t)k * kStat;
       const double2 c = csum[k];
-      gk[0] = l12 * (float)((double)st[1] + (double)st[2] * c.x);
-      gk[1] = l12 * (float)((double)st[6] + (double)st[7] * c.y);
+      gm0 = (double)st[1] + (double)st[2] * c.x;
+      gm1 = (double)st[6] + (double)st[7] * c.y;
       // square-saw drive kappa_k = min(50, 1 + SR/(8 f_k)): d kappa / d m =
       // -(kappa - 1) ln2/12 while below the bound and the pitch is uncapped
       const float kap = buf.kappa[((size_t)v * 2 + 0) * K + k];
       if (kap < (float)kBrightnessMax &&
           !((buf.seg[((size_t)v * 2 + 1) * K + k].jc_flags >> 18) & 1))
-        gk[1] += st[16] * (-(kap - 1.f) * l12);
+        gm1 -= (double)st[16] * (double)(kap - 1.f);
       for (int c3 = 0; c3 < 3; ++c3) gk[2 + c3] = st[10 + c3];
     }
     if (ok && k > 0) {
       const float* st = stat + (size_t)(k - 1) * kStat;
       const double2 c = csum[k - 1];
-      gk[0] += l12 * (float)((double)st[3] + (double)st[4] * c.x);
-      gk[1] += l12 * (float)((double)st[8] + (double)st[9] * c.y);
+      gm0 += (double)st[3] + (double)st[4] * c.x;
+      gm1 += (double)st[8] + (double)st[9] * c.y;
       for (int c3 = 0; c3 < 3; ++c3) gk[2 + c3] += st[13 + c3];
     }
+    gk[0] = (float)(l12 * gm0);
+    gk[1] = (float)(l12 * gm1);
     const float dd[5] = {yv[kSine + 1] * gk[0], gk[2], yv[kSqr + 1] * gk[1], gk[3], gk[4]};
     float dst[5];
     for (int j = 0; j < 5; ++j) dst[j] = buf.dest[((size_t)v * 5 + j) * P + kk];
