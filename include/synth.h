@@ -29,7 +29,13 @@
  *    wave finishes (programmatic dependent launch; the handle alternates two
  *    scratch slots). This is done only when neither launch writes a buffer
  *    the other reads or writes; otherwise, and between a render and any
- *    other kernel, copy or event, stream order holds as usual.
+ *    other kernel, copy or event, stream order holds as usual. That includes
+ *    kernels of other libraries that let their successor start early: a
+ *    render waits for them before it reads given parameters and, where all
+ *    of its tiles fit the GPU at once (86 voices of 4 s), before it writes.
+ *    Only a larger render of drawn parameters writes its buffers while such a
+ *    kernel behind an earlier render may still be reading them: put an event
+ *    between the two.
  */
 #ifndef SYNTH_H
 #define SYNTH_H
