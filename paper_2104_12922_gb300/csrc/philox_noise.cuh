@@ -13,9 +13,11 @@
 // with a bit-identical result.
 //
 // The fractional-rate audio loop of the fused render uses it (3.5% less time
-// per batch at 16 kHz, and that loop no longer spills); the integer-rate loop
+// per batch at 16 kHz, and that loop no longer spills). The integer-rate loop
 // keeps the plain rounds, which measured 1.2% faster there, as did a lighter
-// split that holds only the first three rounds' fixed parts.
+// split that holds only the first three rounds' fixed parts. The normalised
+// renders, at either rate, read the fixed parts from shared memory
+// (philox_noise_shared).
 //
 // Host-compilable (plain C++ outside nvcc) so that a CPU test can compare it
 // with the plain rounds.
@@ -122,14 +124,16 @@ SYNTH_PHILOX_HD void philox_noise(const PhiloxNoise& p, uint32_t q, uint32_t out
 #if defined(__CUDACC__)
 // The same with the fixed parts in shared memory (16-byte aligned), loaded
 // where they are used, four words at a time: held in registers, or left to the
-// compiler to hoist, they spill the render's audio loop.
+// compiler to hoist, they spill the render's audio loop. The loads are marked as
+// reading memory, so that no ordinary store to *p may pass them.
 __device__ __forceinline__ uint4 philox_noise_shared(const PhiloxNoise* p, uint32_t q) {
   const uint32_t at = (uint32_t)__cvta_generic_to_shared(p);
   uint32_t f[4];
   auto fixed = [&](int i) {
     asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
                  : "=r"(f[0]), "=r"(f[1]), "=r"(f[2]), "=r"(f[3])
-                 : "r"(at + 16 * i));
+                 : "r"(at + 16 * i)
+                 : "memory");
   };
   auto product = [](uint32_t m, uint32_t a, uint32_t& hi, uint32_t& lo) {
     hi = __umulhi(m, a);
