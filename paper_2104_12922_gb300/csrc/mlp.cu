@@ -357,6 +357,19 @@ struct LayerGrad {
   float* dzf;
 };
 
+// Joins the side stream to st where a step ends early with an error: what already
+// runs beside it reads the caller's features and writes the weights, and a capture
+// may not end with a forked stream open.
+struct SideJoin {
+  const MlpSide& side;
+  cudaStream_t st;
+  bool open = true;
+  ~SideJoin() {
+    if (open && cudaEventRecord(side.done, side.st) == cudaSuccess)
+      cudaStreamWaitEvent(st, side.done, 0);
+  }
+};
+
 size_t grad_elems(const MlpLayout& L) {
   return (size_t)L.max_batch * (L.dims[1] > L.out_pad ? L.dims[1] : L.out_pad);
 }
@@ -412,6 +425,7 @@ cudaError_t mlp_train_step(const MlpLayout& L, char* base, const MlpSide& side,
   if ((e = cudaEventRecord(side.begun, st)) != cudaSuccess ||
       (e = cudaStreamWaitEvent(side.st, side.begun, 0)) != cudaSuccess)
     return e;
+  SideJoin side_join{side, st};
   {
     dim3 g((L.dims[0] + 31) / 32, (batch + 31) / 32), b(32, 8);
     if ((e = launch_pdl(transpose_bf16, g, b, 0, side.st, x, batch, L.dims[0], h0t)) != cudaSuccess ||
@@ -506,6 +520,7 @@ cudaError_t mlp_train_step(const MlpLayout& L, char* base, const MlpSide& side,
       (e = adam(0, st)) != cudaSuccess ||
       (e = cudaStreamWaitEvent(st, side.done, 0)) != cudaSuccess)
     return e;
+  side_join.open = false;
   return cudaGetLastError();
 }
 

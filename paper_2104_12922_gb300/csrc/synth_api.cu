@@ -555,7 +555,8 @@ synth_status synth_model_train_features(synth_model m, const void* features_dev,
   m->step += 1;
   m->last_batch = batch;
   return check_cuda(mlp_train_step(m->L, m->mem, m->side,
-                                   static_cast<const __nv_bfloat16*>(features_dev), target_dev, batch, lr, m->step, loss_dev, &hdr->error,
+                                   static_cast<const __nv_bfloat16*>(features_dev), target_dev,
+                                   batch, lr, m->step, loss_dev, &hdr->error,
                                    static_cast<cudaStream_t>(stream)));
 }
 
