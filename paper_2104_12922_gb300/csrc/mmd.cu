@@ -22,6 +22,7 @@
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <array>
 #include <climits>
 #include <cstdint>
@@ -59,17 +60,26 @@ namespace {
 // S_i, S_j the two rows' own sums over them formed by the same products, the
 // running FP32 sum takes M - (S_i + S_j) / 2, half the distance over those
 // values. It thus grows like the distance, not like the values, has 690
-// additions at 44160 values instead of 44160 (measured against 64 bits:
-// 2.7e-6 relative before, 3.8e-7 here), and is exactly 0 for equal rows. What
-// the products lose is relative to the rows' sums of absolute values N; where
-// d is below (N_i + N_j) / kCloseRatio, and where a value is not finite, the
-// pair is computed again as written, |a - b| term by term in FP32.
+// additions at 44160 values instead of 44160, and is exactly 0 for equal rows. What
+// the products lose is relative to the rows' sums of absolute values, N = N_i + N_j:
+// at most 28 2^-24 N, so 28 2^-24 N / d of d. A sum of |a - b| term by term in FP32
+// loses at most dim 2^-24 of d. So a pair goes through the maxima where
+// N / d <= dim / 128, at most kCloseRatio (a bound of 4.3e-4 of d then, from dim =
+// 32768 on; 1.3e-5 at 1024), and is computed again term by term beyond, as where a
+// value is not finite. The line is where the errors of unrelated, shifted and heavy-
+// tailed rows meet those of the term-by-term sum in order: root mean square against
+// 64 bits, heavy-tailed rows, maxima / in order: 1024 values, N / d = 8.6: 9.3e-8 /
+// 1.4e-7, 16: 1.3e-7 / 1.1e-7; 2816, 16: 1.3e-7 / 2.4e-7, 32: 2.0e-7 / 1.8e-7; 44160,
+// 1.1: 1.0e-7 / 3.1e-6, 231: 6.4e-7 / 1.0e-6. Below kTermsDim values the maxima would
+// pay for few pairs, and every tile is computed term by term: 3000 sounds of 512
+// values 206 us (maxima and then terms for most tiles 380), of 128 values 65 (74).
 constexpr int kDT = 64;            // distance tile (rows and columns)
 constexpr int kDK = 128;           // embedding values per stage
 constexpr int kDStages = 3;
 constexpr int kDThreads = 512;
 constexpr int kMaxCluster = 8;
-constexpr float kCloseRatio = 256.f;
+constexpr float kCloseRatio = 256.f, kDimPerRatio = 128.f;
+constexpr int kTermsDim = 1024;
 constexpr int kListed = 512;       // close pairs of a tile computed one by one; more: the whole tile
 
 struct L1Smem {
@@ -148,13 +158,15 @@ __device__ __forceinline__ void l1_commit() { asm volatile("cp.async.commit_grou
 __device__ __forceinline__ void l1_wait() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 __device__ __forceinline__ void l1_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// The tile's distances term by term: thread t takes rows 2 (t / 16) + {0, 1}
-// and columns t % 16 + 16 {0..3}.
+// The tile's distances term by term. Two groups of 256 threads take half of the
+// values each (every other 16-byte chunk); thread t of a group has rows
+// t / 16 + 16 {0..3} and columns t % 16 + 16 {0..3}. The halves are then added, and
+// the tile and its mirror written row by row.
 __device__ __noinline__ void l1_tile_by_terms(L1Smem& s, const __nv_bfloat16* emb, int64_t ld,
                                               int m, int dim, int r0, int c0, float* dist) {
   const int n_chunks = (dim + kDK - 1) / kDK;
-  const int ti = 2 * (threadIdx.x >> 4), tj = threadIdx.x & 15;
-  float acc[2][4] = {};
+  const int group = threadIdx.x >> 8, ti = (threadIdx.x >> 4) & 15, tj = threadIdx.x & 15;
+  float acc[4][4] = {};
   __syncthreads();
   l1_load(s, 0, 0, emb, ld, m, dim, r0, c0);
   l1_commit();
@@ -166,37 +178,51 @@ __device__ __noinline__ void l1_tile_by_terms(L1Smem& s, const __nv_bfloat16* em
     if (c + 2 < n_chunks) l1_load(s, (c + 2) % kDStages, c + 2, emb, ld, m, dim, r0, c0);
     l1_commit();
     const auto& st = s.stage[c % kDStages];
-#pragma unroll 2
-    for (int ch = 0; ch < kDK / 8; ++ch) {
-      uint4 a[2];
-#pragma unroll
-      for (int p = 0; p < 2; ++p) a[p] = st[ti + p][l1_chunk(ti + p, ch)];
+#pragma unroll 1
+    for (int ch = group; ch < kDK / 8; ch += 2) {
+      uint4 b[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int row = kDT + tj + 16 * q;
-        const uint4 b = st[row][l1_chunk(row, ch)];
+        b[q] = st[row][l1_chunk(row, ch)];
+      }
 #pragma unroll
-        for (int p = 0; p < 2; ++p) acc[p][q] = add_abs_diff8(acc[p][q], a[p], b);
+      for (int p = 0; p < 4; ++p) {
+        const int row = ti + 16 * p;
+        const uint4 a = st[row][l1_chunk(row, ch)];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[p][q] = add_abs_diff8(acc[p][q], a, b[q]);
       }
     }
   }
+  l1_wait_all();
+  __syncthreads();
+  using Part = float[kDT][kDT + 1];
+  static_assert(2 * sizeof(Part) <= sizeof(s.stage), "the halves fit the stages");
+  Part* part = reinterpret_cast<Part*>(&s.stage[0][0][0]);
 #pragma unroll
-  for (int p = 0; p < 2; ++p)
+  for (int p = 0; p < 4; ++p)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int i = r0 + ti + p, j = c0 + tj + 16 * q;
-      if (i < m && j < m) {
-        dist[(int64_t)i * m + j] = acc[p][q];
-        dist[(int64_t)j * m + i] = acc[p][q];
-      }
-    }
+    for (int q = 0; q < 4; ++q) part[group][ti + 16 * p][tj + 16 * q] = acc[p][q];
+  __syncthreads();
+  for (int e = threadIdx.x; e < kDT * kDT; e += kDThreads) {
+    const int i = e / kDT, j = e % kDT;
+    const float d = part[0][i][j] + part[1][i][j];
+    part[0][i][j] = d;
+    if (r0 + i < m && c0 + j < m) dist[(int64_t)(r0 + i) * m + c0 + j] = d;
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < kDT * kDT; e += kDThreads) {
+    const int j = e / kDT, i = e % kDT;
+    if (r0 + i < m && c0 + j < m) dist[(int64_t)(c0 + j) * m + r0 + i] = part[0][i][j];
+  }
 }
 
 // A cluster of CTAs (1 to 8) shares a tile: each takes a part of the chunks,
 // and the first adds their sums in rank order.
 __global__ void __launch_bounds__(kDThreads, 1)
     l1_distance_kernel(const __nv_bfloat16* __restrict__ emb, int64_t ld, int m, int dim,
-                       float* __restrict__ dist) {
+                       float* __restrict__ dist, float close_ratio) {
   extern __shared__ __align__(16) unsigned char l1_smem[];
   L1Smem& s = *reinterpret_cast<L1Smem*>(l1_smem);
   const cg::cluster_group cluster = cg::this_cluster();
@@ -210,6 +236,10 @@ __global__ void __launch_bounds__(kDThreads, 1)
   while ((r + 1) * (r + 2) / 2 <= t) ++r;
   const int bi = nb - 1 - r, bj = nb - 1 - (t - r * (r + 1) / 2);
   const int r0 = bi * kDT, c0 = bj * kDT;
+  if (dim < kTermsDim) {  // one CTA a tile
+    l1_tile_by_terms(s, emb, ld, m, dim, r0, c0, dist);
+    return;
+  }
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, q = lane & 3;
@@ -302,7 +332,7 @@ __global__ void __launch_bounds__(kDThreads, 1)
       for (int u = 0; u < 2; ++u)
 #pragma unroll
         for (int jj = 0; jj < 4; ++jj)
-          close += !(2.f * kCloseRatio * run[u][jj] >=
+          close += !(2.f * close_ratio * run[u][jj] >=
                      s.norm[wi + 4 * u + q] + s.norm[kDT + wj + 8 * jj + g]);
       if (__syncthreads_count(close > 4) > kDThreads / 2) {
         by_terms = true;
@@ -348,7 +378,7 @@ __global__ void __launch_bounds__(kDThreads, 1)
         if (i > j || j >= m) continue;
         const float d = 2.f * run[u][jj];
         const float n = s.norm[li] + s.norm[kDT + lj];
-        if (!((i == j || kCloseRatio * d >= n) && n < 1e37f)) {
+        if (!((i == j || close_ratio * d >= n) && n < 1e37f)) {
           const int at = atomicAdd(&s.n_close, 1);
           if (at < kListed) s.close[at] = (uint16_t)(li * kDT + lj);
         }
@@ -510,7 +540,7 @@ cudaError_t launch_l1_distances(const __nv_bfloat16* emb, int64_t ld, int m, int
   int best = 1;
   double best_t = 0.0;
   for (int n = 1, l = 0; n <= kMaxCluster; n *= 2, ++l) {
-    if (held[l] < 1 || (n > 1 && n_chunks < 4 * n)) continue;
+    if (held[l] < 1 || (n > 1 && (n_chunks < 4 * n || dim < kTermsDim))) continue;
     const double waves = (double)((tiles + held[l] - 1) / held[l]);
     const double t = waves * ((double)n_chunks / n + (n > 1 ? 4.0 : 0.0));
     if (best_t == 0.0 || t < best_t) { best = n; best_t = t; }
@@ -518,7 +548,8 @@ cudaError_t launch_l1_distances(const __nv_bfloat16* emb, int64_t ld, int m, int
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[1];
   l1_config(cfg, at, best, tiles, st);
-  return cudaLaunchKernelEx(&cfg, l1_distance_kernel, emb, ld, m, dim, dist);
+  const float close_ratio = std::min(kCloseRatio, (float)dim / kDimPerRatio);  // see Precision above
+  return cudaLaunchKernelEx(&cfg, l1_distance_kernel, emb, ld, m, dim, dist, close_ratio);
 }
 
 cudaError_t launch_mmd_trials(const float* dist, int m, const int8_t* labels, int trials,
