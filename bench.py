@@ -530,8 +530,9 @@ def mmd_leg(pkg, torch, dev, num_sms: int, sm_mhz: float, per_corpus: int = 1024
     syn.close()
     dim = emb.shape[1]
     pair_elems = m * (m + 1) / 2 * dim  # upper triangle incl. the diagonal tiles' halves
-    # FP32 pipe: 128 lanes per SM per clock, 2 instructions per element pair
-    peak = num_sms * 128 * sm_mhz * 1e6 / 2
+    # instruction issue: 12 slots of a scheduler per 256 element pairs (four packed
+    # maxima of 64 pairs, one tensor-core product that holds it for eight)
+    peak = num_sms * 4 * sm_mhz * 1e6 * 256 / 12
     return {"corpora": {nm: per_corpus for nm in names}, "n_per_set": n, "trials_per_pair": trials,
             "embedding": "log-mel features (345 frames x 128 bands, bf16), l1 distance",
             "mmd": {f"{names[a]}/{names[b]}": {"mean": float(mm[i].mean()),
@@ -539,11 +540,11 @@ def mmd_leg(pkg, torch, dev, num_sms: int, sm_mhz: float, per_corpus: int = 1024
                     for i, (a, b) in enumerate(pairs)},
             "distance_matrix": {"m": m, "ms": dist_ms,
                                 "g_pair_elements_per_s": pair_elems / (dist_ms / 1e3) / 1e9,
-                                "roofline": {"bound": "alu", "peak_g_per_s": peak / 1e9,
+                                "roofline": {"bound": "issue", "peak_g_per_s": peak / 1e9,
                                              "frac": pair_elems / (dist_ms / 1e3) / peak,
-                                             "peak_source": f"{num_sms} SMs x 128 FP32 lanes x "
-                                                            f"{sm_mhz:.0f} MHz / 2 instructions "
-                                                            "per element pair"}},
+                                             "peak_source": f"{num_sms} SMs x 4 schedulers x "
+                                                            f"{sm_mhz:.0f} MHz x 256 element "
+                                                            "pairs / 12 issue slots"}},
             "trials_ms": trials_ms}
 
 

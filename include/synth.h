@@ -278,7 +278,9 @@ synth_status synth_mrstft(synth_handle h, const float* x_dev, const float* y_dev
  * synth_l1_distances: the pooled distance matrix dist_dev [m][m] FP32,
  * dist[i][j] = sum_k |e_i[k] - e_j[k]| over the rows of emb_dev [m][ld]
  * (bf16, row stride ld elements: a multiple of 8 and >= dim; 16-byte
- * aligned base), FP32 sums on the CUDA cores; symmetric, zero diagonal.
+ * aligned base), FP32 sums; symmetric, zero diagonal. The error is not above
+ * that of |a - b| added up in order in FP32: pairs of long rows that are not
+ * close go through exact maxima, 2 max(a, b) - a - b, the others term by term.
  * Errors: SYNTH_ERR_ARG (bad sizes or pointers), SYNTH_ERR_CUDA. */
 synth_status synth_l1_distances(synth_handle h, const void* emb_dev, int64_t ld, int32_t m,
                                 int32_t dim, float* dist_dev, void* stream);

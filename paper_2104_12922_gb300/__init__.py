@@ -426,7 +426,7 @@ def render_autograd(synth: "Synth", seed: int, batch_index: int, params):
 
 # ---- spectral distance, refinement and the learned proposal -------------------
 class MRSTFT:
-    """Multi-resolution log-magnitude STFT distance on the tensor cores
+    """Multi-resolution log-magnitude STFT distance, by FP32 FFTs
     (synth_mrstft): per-voice loss and gradient w.r.t. x."""
 
     def __init__(self, synth: Synth, batch: int):
